@@ -55,7 +55,8 @@ struct GemmWork {
   int32_t split;        // K-range split, 1 <= split <= k_blocks
   int32_t k_blocks;     // ceil(K / 64)
   int32_t unit_begin;   // first unit of this GEMM within the launch
-  int32_t c_tma;        // 1: C is written through tmap_c by TMA stores
+  int32_t c_tma;        // C and its rows are 16-byte aligned: 1, written through tmap_c by TMA stores;
+                        // 2, split-K (no map: the reduction stores from registers); 0 not aligned
   int32_t batch;        // strided batch entries (1: a plain GEMM)
 };
 
@@ -165,6 +166,7 @@ __device__ __forceinline__ UnitCoord decode_unit(const LaunchParams<MAXG>& p, in
 // measured ~0.4 us before the first load of a launch.
 struct UnitTable {
   int32_t unit_begin, split, tiles_m, tiles_n, k_blocks;
+  int32_t n;            // columns of C (the pair kernel narrows a last column tile of at most 128)
 };
 
 __device__ __forceinline__ UnitCoord decode_unit_tab(const UnitTable* t, int n_gemms, int u) {
@@ -343,81 +345,295 @@ __device__ __forceinline__ void reduce_slice(const CView& w, const float4* tile_
   }
 }
 
-// Store one accumulator tile (128 rows x MMA_N columns, rows m0.., columns
-// n0..) through shared memory with TMA.  Per chunk of 128-byte rows (32 fp32
-// or 64 bf16 columns) every thread writes its row into a staging buffer with
-// the 128-byte swizzle (so a warp's writes hit distinct banks), then one
-// thread issues the tensor store; two 16 KB buffers alternate, and a buffer
-// is reused only after the store two chunks back has read it.  WIDE: the
-// chunks go to consecutive 16 KB buffers from `staging` on (MMA_N * 512 bytes
-// for fp32, half that for bf16), none reused, and only the staging is done
-// here (shared memory only; issue_tile_wide stores them) — for a CTA's last
-// tile, staged in its idle operand ring.  The store clips rows and columns
-// outside C.
-template <int MMA_N, bool OUT_BF16, bool WIDE = false>
-__device__ __forceinline__ void store_tile_tma(const void* tmap_c, uint32_t staging, uint32_t& stg, uint32_t taddr,
-                                               int r, int et, int m0, int n0, int b) {
-  constexpr int CHUNK = OUT_BF16 ? 64 : 32;
-#pragma unroll 1
-  for (int c0 = 0; c0 < MMA_N; c0 += CHUNK) {
-    const uint32_t buf = WIDE ? staging + uint32_t(c0 / CHUNK) * 16384u : staging + (stg & 1u) * 16384u;
-    if (!WIDE && et == 0) ptx::bulk_wait_group_read<1>();
-    ptx::named_bar_sync(1, 128);
-    const uint32_t row = buf + uint32_t(r) * 128u;
-    const uint32_t sw = uint32_t(r & 7);
-    uint32_t raw[32];
-    __syncwarp();
-    ptx::tmem_ld_32x32b_x32(taddr + c0, raw);
-    ptx::tmem_ld_wait();
-    if (!OUT_BF16) {
+// ---------------------------------------------------------------------------
+// Output through shared memory.
+//
+// The four epilogue warps stage the accumulator tile (128 rows, 32 a warp) in
+// chunks of 128-byte rows (32 fp32 or 64 bf16 columns, 16 KB a chunk) with the
+// 128-byte swizzle, so that a warp's writes spread over all banks.  A chunk
+// then leaves either by one tensor store of all 128 rows (rows and columns
+// outside C are clipped), or, where C's rows are not 16-byte aligned or its
+// columns end inside a 16-byte granule, warp by warp with plain stores, the
+// lanes along the columns.  A warp whose rows lie past M stages nothing.
+//
+// Why one store per 128 rows: four stores of 32 rows without the barriers
+// among the warps cost the copy engine, which the operand loads share, more
+// than the barriers cost (bench set of 280 pair tiles: 50.0 -> 51.1 us).  Why
+// lanes along the columns: one row per lane wrote 4 bytes of each 32-byte
+// sector per instruction (777 x 1501 x 1003, fp32 rows 4-byte aligned: 19.2
+// -> 13.8 us).
+// ---------------------------------------------------------------------------
+constexpr uint32_t kWarpChunk = 4096;    // 32 rows x 128 bytes: a warp's part of a chunk
+constexpr uint32_t kChunkBytes = 16384;  // 128 rows x 128 bytes
+
+// Columns of C per staged chunk.
+template <bool OUT_BF16>
+struct ChunkCols {
+  static constexpr int value = OUT_BF16 ? 64 : 32;
+};
+
+// Stage 32 accumulator columns (fp32 values) of this lane's row: a whole
+// chunk row for fp32, half of one (`half` 0 or 1) for bf16.
+template <bool OUT_BF16>
+__device__ __forceinline__ void stage_cols(uint32_t buf, int lane, int half, const uint32_t (&v)[32]) {
+  const uint32_t row = buf + uint32_t(lane) * 128u;
+  const uint32_t sw = uint32_t(lane & 7);
+  if (!OUT_BF16) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        ptx::st_shared_v4(row + ((uint32_t(j) ^ sw) << 4), raw[4 * j], raw[4 * j + 1], raw[4 * j + 2], raw[4 * j + 3]);
-    } else {
-      uint32_t pk[16];
+    for (int j = 0; j < 8; ++j)
+      ptx::st_shared_v4(row + ((uint32_t(j) ^ sw) << 4), v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+  } else {
+    uint32_t pk[16];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(raw[2 * j]), __uint_as_float(raw[2 * j + 1]));
-        pk[j] = *reinterpret_cast<uint32_t*>(&h);
-      }
-      __syncwarp();
-      ptx::tmem_ld_32x32b_x32(taddr + c0 + 32, raw);
-      ptx::tmem_ld_wait();
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        ptx::st_shared_v4(row + ((uint32_t(j) ^ sw) << 4), pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(raw[2 * j]), __uint_as_float(raw[2 * j + 1]));
-        pk[j] = *reinterpret_cast<uint32_t*>(&h);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        ptx::st_shared_v4(row + ((uint32_t(j + 4) ^ sw) << 4), pk[4 * j], pk[4 * j + 1], pk[4 * j + 2],
-                          pk[4 * j + 3]);
+    for (int j = 0; j < 16; ++j) {
+      __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+      pk[j] = *reinterpret_cast<uint32_t*>(&h);
     }
-    ptx::fence_proxy_async_smem();
-    if (WIDE) continue;
-    ptx::named_bar_sync(1, 128);
-    if (et == 0) {
-      ptx::tma_store_3d(tmap_c, buf, n0 + c0, m0, b);
-      ptx::bulk_commit_group();
-    }
-    ++stg;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      ptx::st_shared_v4(row + ((uint32_t(4 * half + j) ^ sw) << 4), pk[4 * j], pk[4 * j + 1], pk[4 * j + 2],
+                        pk[4 * j + 3]);
   }
-  if (WIDE) ptx::named_bar_sync(1, 128);   // every chunk staged and fenced
 }
 
-// The tensor stores of a tile staged by store_tile_tma<..., true> (one
-// thread issues them all, one bulk group).
+// Stage one chunk straight from tensor memory.
+template <bool OUT_BF16>
+__device__ __forceinline__ void stage_chunk(uint32_t buf, int lane, uint32_t taddr) {
+  uint32_t raw[32];
+  __syncwarp();
+  ptx::tmem_ld_32x32b_x32(taddr, raw);
+  if (OUT_BF16) {
+    uint32_t raw2[32];
+    ptx::tmem_ld_32x32b_x32(taddr + 32, raw2);
+    ptx::tmem_ld_wait();
+    stage_cols<OUT_BF16>(buf, lane, 0, raw);
+    stage_cols<OUT_BF16>(buf, lane, 1, raw2);
+  } else {
+    ptx::tmem_ld_wait();
+    stage_cols<OUT_BF16>(buf, lane, 0, raw);
+  }
+}
+
+// Copy a staged chunk (rows row0 .., columns col0 .. of C) with plain stores,
+// the lanes along the columns: each instruction writes up to 128 contiguous
+// bytes of one row, whatever the row's alignment.
+template <bool OUT_BF16>
+__device__ __forceinline__ void copy_chunk(const CView& w, uint32_t buf, int lane, int row0, int col0) {
+  const int rows = min(32, w.m - row0);
+  const int cols = min(ChunkCols<OUT_BF16>::value, w.n - col0);
+  if (!OUT_BF16) {
+    float* dst = static_cast<float*>(w.c) + int64_t(row0) * w.ldc + col0 + lane;
+    if (lane >= cols) return;
+#pragma unroll 4
+    for (int rr = 0; rr < rows; ++rr) {
+      const uint32_t at = buf + uint32_t(rr) * 128u + ((uint32_t(lane >> 2) ^ uint32_t(rr & 7)) << 4) + (lane & 3) * 4;
+      *dst = __uint_as_float(ptx::ld_shared_u32(at));
+      dst += w.ldc;
+    }
+  } else {
+    // two columns per lane; in a row that starts 2 bytes off a 4-byte
+    // boundary the pairs start at column 1 and the last lane takes the first
+    // and last columns alone
+    __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(w.c) + int64_t(row0) * w.ldc + col0;
+#pragma unroll 4
+    for (int rr = 0; rr < rows; ++rr) {
+      const uint32_t row = buf + uint32_t(rr) * 128u;
+      const uint32_t sw = uint32_t(rr & 7);
+      auto elem = [&](int e) {
+        return ptx::ld_shared_u16(row + ((uint32_t(e >> 3) ^ sw) << 4) + uint32_t(e & 7) * 2u);
+      };
+      uint16_t* d16 = reinterpret_cast<uint16_t*>(dst);
+      if ((reinterpret_cast<uintptr_t>(dst) & 2) == 0) {
+        const int e = 2 * lane;
+        const uint32_t v = ptx::ld_shared_u32(row + ((uint32_t(e >> 3) ^ sw) << 4) + uint32_t(e & 7) * 2u);
+        if (e + 1 < cols)
+          *reinterpret_cast<uint32_t*>(d16 + e) = v;
+        else if (e < cols)
+          d16[e] = uint16_t(v);
+      } else {
+        const int e = 2 * lane + 1;
+        const uint32_t lo = elem(e);
+        const uint32_t hi = elem((e + 1) & 63);   // lane 31: column 0
+        if (lane == 31) {
+          if (e < cols) d16[e] = uint16_t(lo);
+          d16[0] = uint16_t(hi);
+        } else if (e + 1 < cols) {
+          *reinterpret_cast<uint32_t*>(d16 + e) = lo | (hi << 16);
+        } else if (e < cols) {
+          d16[e] = uint16_t(lo);
+        }
+      }
+      dst += w.ldc;
+    }
+  }
+}
+
+// Can the chunk at column col0 leave by a tensor store?  A tensor store
+// writes whole 16-byte granules, so a chunk whose columns end inside one
+// would also write the row's padding past N.
+template <bool OUT_BF16>
+__device__ __forceinline__ bool tma_chunk(const CView& w, bool tma, int col0) {
+  return tma && (w.n - col0 >= ChunkCols<OUT_BF16>::value || w.n % (OUT_BF16 ? 8 : 4) == 0);
+}
+
+// The next of the two staging buffers, once the store two chunks back has
+// read it (all 128 epilogue threads).
+__device__ __forceinline__ uint32_t next_buf(uint32_t staging, uint32_t& stg, int et) {
+  const uint32_t buf = staging + (stg & 1u) * kChunkBytes;
+  ++stg;
+  if (et == 0) ptx::bulk_wait_group_read<1>();
+  ptx::named_bar_sync(1, 128);
+  return buf;
+}
+
+// Send the chunk staged at `buf` to rows m0 .., columns col0 .. of C (all 128
+// epilogue threads).
+template <bool OUT_BF16>
+__device__ __forceinline__ void send_chunk(const CView& w, const void* tmap_c, bool tma, uint32_t buf, int et, int q,
+                                           int m0, int col0, int b) {
+  if (tma_chunk<OUT_BF16>(w, tma, col0)) {
+    ptx::fence_proxy_async_smem();
+    ptx::named_bar_sync(1, 128);
+    if (et == 0) {
+      ptx::tma_store_3d(tmap_c, buf, col0, m0, b);
+      ptx::bulk_commit_group();
+    }
+  } else {
+    // an empty group, so that next_buf's count of the groups in flight stays
+    // the count of chunks
+    if (et == 0) ptx::bulk_commit_group();
+    __syncwarp();
+    if (m0 + 32 * q < w.m) copy_chunk<OUT_BF16>(w, buf + uint32_t(q) * kWarpChunk, et & 31, m0 + 32 * q, col0);
+  }
+}
+
+// Store an accumulator tile of up to MMA_N columns (rows m0 .., columns n0 ..
+// n0 + ncols - 1 of C).  The next chunk's tensor-memory load is issued before
+// this chunk's barrier and store, so its latency is not on the chunk's chain.
 template <int MMA_N, bool OUT_BF16>
-__device__ __forceinline__ void issue_tile_wide(const void* tmap_c, uint32_t staging, int et, int m0, int n0, int b) {
-  constexpr int CHUNK = OUT_BF16 ? 64 : 32;
-  if (et != 0) return;
+__device__ __forceinline__ void store_tile(const CView& w, const void* tmap_c, bool tma, uint32_t staging,
+                                           uint32_t& stg, uint32_t taddr, int et, int q, int m0, int n0, int ncols,
+                                           int b) {
+  constexpr int CHUNK = ChunkCols<OUT_BF16>::value;
+  constexpr int HALVES = CHUNK / 32;
+  constexpr int NCH = MMA_N >= CHUNK ? MMA_N / CHUNK : 1;   // (32-wide transposed kinds never get here)
+  uint32_t raw[NCH][HALVES][32];         // registers: at most one chunk is live at a time
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < HALVES; ++h) ptx::tmem_ld_32x32b_x32(taddr + 32 * h, raw[0][h]);
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    if (i * CHUNK >= ncols) break;
+    const uint32_t buf = next_buf(staging, stg, et);
+    ptx::tmem_ld_wait();
+#pragma unroll
+    for (int h = 0; h < HALVES; ++h) stage_cols<OUT_BF16>(buf + uint32_t(q) * kWarpChunk, et & 31, h, raw[i][h]);
+    if (i + 1 < NCH) {
+      __syncwarp();
+#pragma unroll
+      for (int h = 0; h < HALVES; ++h) ptx::tmem_ld_32x32b_x32(taddr + (i + 1) * CHUNK + 32 * h, raw[i + 1][h]);
+    }
+    send_chunk<OUT_BF16>(w, tmap_c, tma, buf, et, q, m0, n0 + i * CHUNK, b);
+  }
+  ptx::tmem_ld_wait();
+}
+
+// The same in two steps for a CTA's last tile, staged whole in its idle
+// operand ring (chunk c at ring + c * 16 KB): shared memory only, then the
+// stores.
+template <bool OUT_BF16>
+__device__ __forceinline__ void stage_tile_wide(const CView& w, uint32_t ring, uint32_t taddr, int et, int q, int m0,
+                                                int ncols) {
+  if (m0 + 32 * q < w.m)
 #pragma unroll 1
-  for (int c0 = 0; c0 < MMA_N; c0 += CHUNK)
-    ptx::tma_store_3d(tmap_c, staging + uint32_t(c0 / CHUNK) * 16384u, n0 + c0, m0, b);
-  ptx::bulk_commit_group();
+    for (int c0 = 0; c0 < ncols; c0 += ChunkCols<OUT_BF16>::value)
+      stage_chunk<OUT_BF16>(ring + uint32_t(c0 / ChunkCols<OUT_BF16>::value) * kChunkBytes + uint32_t(q) * kWarpChunk,
+                            et & 31, taddr + c0);
+  ptx::fence_proxy_async_smem();
+  ptx::named_bar_sync(1, 128);             // every chunk staged and fenced
+}
+template <bool OUT_BF16>
+__device__ __forceinline__ void send_tile_wide(const CView& w, const void* tmap_c, bool tma, uint32_t ring, int et,
+                                               int q, int m0, int n0, int ncols, int b) {
+  constexpr int CHUNK = ChunkCols<OUT_BF16>::value;
+  if (et == 0) {
+#pragma unroll 1
+    for (int c0 = 0; c0 < ncols; c0 += CHUNK)
+      if (tma_chunk<OUT_BF16>(w, tma, n0 + c0))
+        ptx::tma_store_3d(tmap_c, ring + uint32_t(c0 / CHUNK) * kChunkBytes, n0 + c0, m0, b);
+    ptx::bulk_commit_group();
+  }
+  __syncwarp();
+  if (m0 + 32 * q < w.m)
+#pragma unroll 1
+    for (int c0 = tma ? ncols / CHUNK * CHUNK : 0; c0 < ncols; c0 += CHUNK)
+      if (!tma_chunk<OUT_BF16>(w, tma, n0 + c0))
+        copy_chunk<OUT_BF16>(w, ring + uint32_t(c0 / CHUNK) * kChunkBytes + uint32_t(q) * kWarpChunk, et & 31,
+                             m0 + 32 * q, n0 + c0);
+}
+
+// Split-K, last split to arrive: sum the S partials of the tile in split order
+// 0, 1, ..., S-1 and store them.  `parts`: this lane's row of the
+// tile's first partial (layout [column / 4][row]), partial s `stride` float4
+// further on; the own split's values come from tensor memory.  Two splits'
+// partials are loaded before either is added, so their loads are in flight
+// together.  The sums leave through the staging buffers, the lanes along the
+// columns: for C whose rows are not 16-byte aligned (aligned rows are stored
+// from registers, which measured 3% faster on a set of split-K GEMMs).
+template <bool OUT_BF16>
+__device__ __forceinline__ void sum_and_store_tile(const CView& w, const float4* parts, int stride, int S, int own_s,
+                                                   uint32_t staging, uint32_t& stg, uint32_t taddr, int et, int q,
+                                                   int m0, int n0, int ncols) {
+  const bool live = m0 + 32 * q < w.m;
+#pragma unroll 1
+  for (int c0 = 0; c0 < ncols; c0 += ChunkCols<OUT_BF16>::value) {
+    const uint32_t buf = next_buf(staging, stg, et);
+#pragma unroll 1
+    for (int h = 0; h < (OUT_BF16 ? 2 : 1) && live; ++h) {
+      const int cc = c0 + 32 * h;
+      if (cc >= ncols) break;             // the chunk's second half lies past N (its columns are clipped)
+      uint32_t raw[32];
+      __syncwarp();
+      ptx::tmem_ld_32x32b_x32(taddr + cc, raw);
+      ptx::tmem_ld_wait();
+      float v[32];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = 0.0f;
+#pragma unroll 1
+      for (int s2 = 0; s2 < S; s2 += 2) {
+        const bool has_b = s2 + 1 < S;
+        float4 ta[8], tb[8];
+        const float4* pa = parts + size_t(s2) * stride + size_t(cc / 4) * 128;
+#pragma unroll
+        for (int j4 = 0; j4 < 8; ++j4) {
+          const float4 own = make_float4(__uint_as_float(raw[4 * j4]), __uint_as_float(raw[4 * j4 + 1]),
+                                         __uint_as_float(raw[4 * j4 + 2]), __uint_as_float(raw[4 * j4 + 3]));
+          ta[j4] = (s2 == own_s) ? own : __ldcg(&pa[j4 * 128]);
+          tb[j4] = (!has_b || s2 + 1 == own_s) ? own : __ldcg(&pa[size_t(stride) + j4 * 128]);
+        }
+#pragma unroll
+        for (int j4 = 0; j4 < 8; ++j4) {
+          v[4 * j4] += ta[j4].x;
+          v[4 * j4 + 1] += ta[j4].y;
+          v[4 * j4 + 2] += ta[j4].z;
+          v[4 * j4 + 3] += ta[j4].w;
+        }
+        if (has_b) {
+#pragma unroll
+          for (int j4 = 0; j4 < 8; ++j4) {
+            v[4 * j4] += tb[j4].x;
+            v[4 * j4 + 1] += tb[j4].y;
+            v[4 * j4 + 2] += tb[j4].z;
+            v[4 * j4 + 3] += tb[j4].w;
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 32; ++j) raw[j] = __float_as_uint(v[j]);
+      stage_cols<OUT_BF16>(buf + uint32_t(q) * kWarpChunk, et & 31, h, raw);
+    }
+    send_chunk<OUT_BF16>(w, nullptr, false, buf, et, q, m0, n0 + c0, 0);
+  }
 }
 
 // Shared-memory layout of a whole fp32 partial tile for the on-chip cluster
@@ -655,6 +871,7 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
       e.tiles_m = p.g[g].tiles_m;
       e.tiles_n = p.g[g].tiles_n;
       e.k_blocks = p.g[g].k_blocks;
+      e.n = p.g[g].n;
       utab[g] = e;
     }
   }
@@ -897,26 +1114,27 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
       const int m0 = c.tm * TILE_M;
       const int n0 = c.tn * TILE_N;
       const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(acc * MMA_N);
-      // this CTA's last tile with nothing but tensor stores: the operand
-      // ring is idle (every MMA done, no load left) and stages all of it
-      // (two-per-SM kinds too, where their ring holds the tile: they keep no
-      // staging buffers and store their other tiles directly)
+      // this CTA's last tile: the operand ring is idle (every MMA done, no
+      // load left) and stages all of it, so that only its stores follow the
+      // wait for the previous grid (two-per-SM kinds too, where their ring
+      // holds the tile: they keep no staging buffers and store their other
+      // tiles directly)
       static_assert(!EPI_TMA || kWideFits, "the ring holds a whole tile");
-      const bool wide = kWideFits && w.split == 1 && w.c_tma && p.dyn == nullptr &&
-                        u + int(gridDim.x) >= p.total_units;
+      const bool wide = kWideFits && w.split == 1 && p.dyn == nullptr && u + int(gridDim.x) >= p.total_units;
+      const int ncols = min(MMA_N, w.n - n0);
       // the cluster reductions on chip exchange partials through shared
       // memory only and wait just before their stores
       const bool onchip = kPartFitsRing && p.cluster > 0 && p.total_units == int(gridDim.x);
       if (wide) {
-        store_tile_tma<MMA_N, OUT_BF16, true>(&p.tmap_c[c.g], tiles_base, stg, taddr, r, et, m0, n0, c.b);
+        stage_tile_wide<OUT_BF16>(cv, tiles_base, taddr, et, q, m0, ncols);
         wait_prev();
-        issue_tile_wide<MMA_N, OUT_BF16>(&p.tmap_c[c.g], tiles_base, et, m0, n0, c.b);
+        send_tile_wide<OUT_BF16>(cv, &p.tmap_c[c.g], w.c_tma != 0, tiles_base, et, q, m0, n0, ncols, c.b);
       } else if (!(w.split > 1 && (push_on || onchip))) {
         wait_prev();
       }
       if (wide) {
-      } else if (EPI_TMA && w.split == 1 && w.c_tma) {
-        store_tile_tma<MMA_N, OUT_BF16>(&p.tmap_c[c.g], staging, stg, taddr, r, et, m0, n0, c.b);
+      } else if (EPI_TMA && w.split == 1) {
+        store_tile<MMA_N, OUT_BF16>(cv, &p.tmap_c[c.g], w.c_tma != 0, staging, stg, taddr, et, q, m0, n0, ncols, c.b);
       } else if (w.split == 1) {
 #pragma unroll 1
         for (int c0 = 0; c0 < MMA_N; c0 += 32) {
@@ -1091,8 +1309,12 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
         ptx::named_bar_sync(1, 128);
         if (*last_flag) {
           __threadfence();
+          const bool staged = EPI_TMA && w.c_tma == 0;
+          if (staged)
+            sum_and_store_tile<OUT_BF16>(cv, part_base + size_t(c.tile * w.split) * TILE_F4 + r, TILE_F4, w.split, c.s,
+                                         staging, stg, taddr, et, q, m0, n0, ncols);
 #pragma unroll 1
-          for (int c0 = 0; c0 < MMA_N; c0 += 32) {
+          for (int c0 = 0; c0 < (staged ? 0 : MMA_N); c0 += 32) {
             uint32_t raw[32];
             __syncwarp();
             ptx::tmem_ld_32x32b_x32(taddr + c0, raw);

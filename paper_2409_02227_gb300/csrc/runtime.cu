@@ -414,12 +414,14 @@ goldy_status fill_slot(LaunchParams<MAXG>& p, int j, const GemmPlan& gp, const v
   // idle operand ring)
   w.c_tma = 0;
   const uint64_t sc = uint64_t(w.c_bstride) * es;
-  if (!k.swap_ab && gp.split == 1 && aligned(C, 16) && (size_t(g.ldc) * es) % 16 == 0 && sc % 16 == 0) {
-    st = encode_3d(&p.tmap_c[j], C, uint64_t(g.N), uint64_t(g.M), uint64_t(g.batch), uint64_t(g.ldc) * es, sc,
-                   uint32_t(128 / es), 128,
-                   g.c_dtype == GOLDY_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32);
-    if (st != GOLDY_OK) return st;
-    w.c_tma = 1;
+  if (!k.swap_ab && aligned(C, 16) && (size_t(g.ldc) * es) % 16 == 0 && sc % 16 == 0) {
+    w.c_tma = gp.split == 1 ? 1 : 2;
+    if (w.c_tma == 1) {
+      st = encode_3d(&p.tmap_c[j], C, uint64_t(g.N), uint64_t(g.M), uint64_t(g.batch), uint64_t(g.ldc) * es, sc,
+                     uint32_t(128 / es), 128,
+                     g.c_dtype == GOLDY_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32);
+      if (st != GOLDY_OK) return st;
+    }
   }
   if (gp.split > 1) {
     w.ws_part = reinterpret_cast<float*>(ws + gp.ws_part_off);
