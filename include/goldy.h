@@ -100,19 +100,24 @@ typedef struct goldy_graph goldy_graph;
 #define GOLDY_PLAN_DEFAULT 2
 #define GOLDY_PLAN_GO 3
 #define GOLDY_PLAN_FORCE_CD 4
-/* Launch-mode bit, combinable with any policy above.  FUSED: within each
- * group, the GEMMs that run at the same time (a "wave" of CD members) and
- * share a kernel kind and output dtype go into ONE persistent launch over the
- * concatenation of their tiles (at most 16 GEMMs per launch); its grid cap is
- * the sum of the members' caps.  A wave's launches carry launch priorities
- * ranked by their FLOPs, and the first wave's largest launch goes out first
- * (outside a stream capture the other streams also wait until all of its
- * CTAs have begun).  Groups are not separated by a join: the run forks once
- * and joins once, and a later group's launches take lower priorities, so they
- * fill the SMs an earlier group frees.  A fused run with
- * goldy_run_opts.inputs_ready = 1 goes out on streams[0] alone
- * instead, each wave's largest launch first, every launch overlapping the
- * previous one's tail (no fork, no join).  Without FUSED every GEMM is its own
+/* Launch-mode bit, combinable with any policy above.  FUSED with AUTO: a plan
+ * whose waves (a group's members taken CD at a time) would need several
+ * launches runs as one persistent launch of the CTA-pair kind's GEMMs and one
+ * of all other kinds' (per output dtype, at most 16 GEMMs per launch), their
+ * tiles dealt out to the GPU's CTAs in equal shares, longest first; both go
+ * out on streams[0] alone, the largest first, each overlapping the previous
+ * one's tail (no fork, no join).  FUSED otherwise (explicit schedules, the
+ * forced policies), and for a plan of a single launch: within each group, the
+ * GEMMs of a wave that share a kernel kind and output dtype go into ONE
+ * persistent launch over the concatenation of their tiles (at most 16 GEMMs
+ * per launch); its grid cap is the sum of the members' caps.  A wave's
+ * launches carry launch priorities ranked by their FLOPs, and the first wave's
+ * largest launch goes out first (outside a stream capture the other streams
+ * also wait until all of its CTAs have begun).  Groups are not separated by a
+ * join: the run forks once and joins once, and a later group's launches take
+ * lower priorities, so they fill the SMs an earlier group frees.  Such a run
+ * with goldy_run_opts.inputs_ready = 1 goes out on streams[0] alone instead,
+ * each wave's largest launch first.  Without FUSED every GEMM is its own
  * launch on its slot's stream and the groups run one after another.  The plan
  * (groups, CDs, variants, slots) is the same, and so are the results, byte
  * for byte. */
@@ -248,7 +253,7 @@ goldy_status goldy_schedule_build(const goldy_gemm_desc* descs, int n, const int
 
 /* Sizes of a schedule.  workspace_bytes is the device workspace goldy_run
  * needs (split-K partial tiles and arrival counters, and for GOLDY_PLAN_FUSED
- * schedules of several GEMMs 8 bytes of unit counters per GEMM; 0 if none). */
+ * schedules of several GEMMs 8 reserved bytes per GEMM; 0 if none). */
 goldy_status goldy_schedule_query(const goldy_schedule* s, int* n_gemms, int* n_groups,
                                   int* max_streams, size_t* workspace_bytes);
 
@@ -279,9 +284,8 @@ void goldy_schedule_free(goldy_schedule* s);
  * misaligned pointers, too few streams, workspace too small),
  * GOLDY_ERR_CUDA (launch failure).  A kernel that gave up a bounded wait
  * shows up later through goldy_device_error(); the outputs of that run are
- * then incomplete, and its workspace may hold non-zero split-K arrival or
- * unit counters: zero-fill the workspace again before the next run that uses
- * it. */
+ * then incomplete, and its workspace may hold non-zero split-K arrival
+ * counters: zero-fill the workspace again before the next run that uses it. */
 goldy_status goldy_run(const goldy_schedule* s, const void* const* A, const void* const* B,
                        void* const* C, void* workspace, size_t workspace_bytes,
                        void* const* streams, int n_streams);
@@ -313,7 +317,10 @@ typedef struct goldy_run_opts {
    * memory, descriptor prefetch) while the previous kernel on its stream is
    * still running — programmatic dependent launch; the kernel waits for that
    * kernel to complete before it touches global memory, so results and
-   * stream order are unchanged.  1: plain serialised launches. */
+   * stream order are unchanged.  (The later launches of a fused AUTO run may
+   * read A and B once the work before the run is complete, while the run's
+   * first launch is still going on; not in a run that traces or sets
+   * wait_limit_us.)  1: plain serialised launches. */
   int32_t serial_launch;
   /* 0 (default): as above.  1: the caller asserts that no kernel enqueued
    * before this run (on its streams) writes any A or B of the run.  Each

@@ -23,7 +23,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libgoldy.so")
-NUM_KINDS = 11
+NUM_KINDS = 12          # 11 kinds and the kernel that mixes their tile shapes
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

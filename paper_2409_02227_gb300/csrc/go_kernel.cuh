@@ -9,8 +9,9 @@
 //
 // How (Sec. 2.1.3's tiled GEMM re-expressed for tcgen05):
 //   * The output is cut into tiles; a tile with its K-range split is a
-//     "unit".  CTA b processes units b, b + gridDim.x, ... (persistent CTAs,
-//     a static round-robin that is a function of the variant only).  The
+//     "unit".  Persistent CTAs: with one GEMM per launch CTA b processes units
+//     b, b + gridDim.x, ...; over several GEMMs every CTA gets an equal share
+//     of the work, dealt out by the host longest units first.  The
 //     grid size is the variant's resource constraint: capping it is how a
 //     GO-Kernel leaves SMs to co-running GEMMs (Sec. 4.2.1).
 //   * warp 0 (one thread): TMA producer.  Per 64-wide K block it loads the
@@ -58,6 +59,7 @@ struct GemmWork {
   int32_t c_tma;        // C and its rows are 16-byte aligned: 1, written through tmap_c by TMA stores;
                         // 2, split-K (no map: the reduction stores from registers); 0 not aligned
   int32_t batch;        // strided batch entries (1: a plain GEMM)
+  int32_t mma_n, swap;  // the tile shape (KindInfo), for launches that mix kinds
 };
 
 // Where one batch entry's C lives: the store helpers' view of a GemmWork.
@@ -77,6 +79,26 @@ __device__ __forceinline__ CView c_view(const GemmWork& w, int b) {
   return v;
 }
 
+// Shares of a launch over several GEMMs: of GEMM g, bin b (a CTA, or a CTA
+// pair) takes units b, b + bins, ... for the rounds[g] rounds that every bin
+// takes part in, then units first[g][b] .. first[g][b + 1] - 1 behind those.
+// The host deals the units out, longest GEMMs first, so that every bin gets
+// the same work (assign_units); with one GEMM per launch the units are equal
+// and go round-robin.  (Whole rounds keep the bins on neighbouring tiles:
+// with one contiguous range per bin the operand panels in use at a time are
+// three times as many, bench set 50.4 -> 51.4 us.)
+constexpr int kMaxBins = 160;
+template <int MAXG>
+struct UnitShares {
+  int32_t on;
+  uint16_t rounds[MAXG];
+  uint16_t first[MAXG][kMaxBins + 1];
+};
+template <>
+struct UnitShares<1> {
+  int32_t on;
+};
+
 template <int MAXG>
 struct LaunchParams {
   CUtensorMap tmap_a[MAXG];   // A: dims {K, M, batch}, box {64, rows of the A tile, 1}
@@ -89,9 +111,6 @@ struct LaunchParams {
   unsigned long long* trace;  // optional phase trace, kTracePerCta stamps per CTA (null: off)
   int32_t cluster;            // 0, or the split-K factor S of every GEMM in the launch when the
                               // launch is made of clusters of S CTAs (the splits of one tile)
-  uint32_t* dyn;              // null: CTA b takes units b, b + grid, ...; else a zeroed pair of
-                              // counters (units taken, CTAs done): after its first unit b a CTA
-                              // takes grid + (counter++), and the last CTA to leave zeroes both
   uint64_t wait_ns;           // limit of every bounded wait (0: ptx::kWaitLimitNs)
   int32_t early_loads;        // 1: the load and MMA roles start before the previous kernel on the
                               // stream has completed (the caller asserted that no earlier kernel
@@ -99,13 +118,12 @@ struct LaunchParams {
                               // touched only after it (griddepcontrol.wait in the epilogue)
   int32_t stall_test;         // test hook: CTA 0's producer never fills its first stage, so the
                               // MMA thread's bounded wait for it runs out (0 in normal use)
+  int32_t late_trigger;       // 1: let the next launch on the stream start only once this one is past its wait
+                              // for the grid before (early_loads is 0 then): the next launch, of the same run,
+                              // may then load its A and B at once, since every grid before the run has completed
+  int32_t stage_bytes, stages;   // operand ring of a launch that mixes tile shapes
+  UnitShares<MAXG> shares;    // on: the units of each CTA (pair); off: round-robin
 };
-
-// Units a CTA has taken but its MMA thread and epilogue have not yet both
-// read, at most (a ring of unit indices in shared memory, used when the
-// launch hands units out from a counter; with the static round-robin every
-// role computes the sequence itself).
-constexpr int kUnitRing = 8;
 
 // Phase trace (optional, for profiling): %globaltimer stamps per CTA.
 enum : int {
@@ -139,55 +157,101 @@ struct UnitCoord {
   int g, tile, s, b, tm, tn, kb0, kb1;   // tile counts over all batch entries; b = batch entry
 };
 
-template <int MAXG>
-__device__ __forceinline__ UnitCoord decode_unit(const LaunchParams<MAXG>& p, int u) {
-  UnitCoord c;
-  int g = 0;
-#pragma unroll 1
-  while (g + 1 < p.n_gemms && u >= p.g[g + 1].unit_begin) ++g;
-  const GemmWork& w = p.g[g];
-  const int local = u - w.unit_begin;
-  c.g = g;
-  c.tile = local / w.split;
-  c.s = local - c.tile * w.split;
-  const int per_batch = w.tiles_m * w.tiles_n;
-  c.b = c.tile / per_batch;
-  const int t = c.tile - c.b * per_batch;
-  c.tm = t % w.tiles_m;
-  c.tn = t / w.tiles_m;
-  c.kb0 = (c.s * w.k_blocks) / w.split;
-  c.kb1 = ((c.s + 1) * w.k_blocks) / w.split;
-  return c;
-}
-
-// The fields of a GemmWork that decode a unit, copied into shared memory at
-// set-up: the kernel parameter block is several kilobytes (tensor maps
-// first), and reading these fields from it on the producer's critical path
-// measured ~0.4 us before the first load of a launch.
+// The fields of a GemmWork that decode a unit, and the units of it that this
+// CTA (pair) takes, copied into shared memory at set-up: the kernel parameter
+// block is several kilobytes (tensor maps first), and reading these fields
+// from it on the producer's critical path measured ~0.4 us before the first
+// load of a launch.
 struct UnitTable {
   int32_t unit_begin, split, tiles_m, tiles_n, k_blocks;
   int32_t n;            // columns of C (the pair kernel narrows a last column tile of at most 128)
+  int32_t rounds, lo, hi;   // this CTA's (pair's) units of the GEMM, when the launch has shares
+  int32_t mma_n, swap;  // tile shape (launches that mix tile shapes)
 };
 
-__device__ __forceinline__ UnitCoord decode_unit_tab(const UnitTable* t, int n_gemms, int u) {
-  UnitCoord c;
-  int g = 0;
-#pragma unroll 1
-  while (g + 1 < n_gemms && u >= t[g + 1].unit_begin) ++g;
-  const UnitTable& w = t[g];
-  const int local = u - w.unit_begin;
-  c.g = g;
-  c.tile = local / w.split;
-  c.s = local - c.tile * w.split;
-  const int per_batch = w.tiles_m * w.tiles_n;
-  c.b = c.tile / per_batch;
-  const int t2 = c.tile - c.b * per_batch;
-  c.tm = t2 % w.tiles_m;
-  c.tn = t2 / w.tiles_m;
-  c.kb0 = (c.s * w.k_blocks) / w.split;
-  c.kb1 = ((c.s + 1) * w.k_blocks) / w.split;
-  return c;
+// Fill the table (one warp).
+template <int MAXG>
+__device__ __forceinline__ void fill_unit_table(UnitTable* t, const LaunchParams<MAXG>& p, int bin, int lane) {
+  for (int g = lane; g < p.n_gemms; g += 32) {
+    UnitTable e;
+    e.unit_begin = p.g[g].unit_begin;
+    e.split = p.g[g].split;
+    e.tiles_m = p.g[g].tiles_m;
+    e.tiles_n = p.g[g].tiles_n;
+    e.k_blocks = p.g[g].k_blocks;
+    e.n = p.g[g].n;
+    e.rounds = e.lo = e.hi = 0;
+    if constexpr (MAXG > 1) {
+      if (p.shares.on) {
+        e.rounds = int(p.shares.rounds[g]);
+        e.lo = e.unit_begin + int(p.shares.first[g][bin]);
+        e.hi = e.unit_begin + int(p.shares.first[g][bin + 1]);
+      }
+    }
+    e.mma_n = p.g[g].mma_n;
+    e.swap = p.g[g].swap;
+    t[g] = e;
+  }
 }
+
+// The sequence of units of one CTA (pair): its shares GEMM by GEMM, or
+// bin, bin + bins, ...  Every role walks its own copy.
+struct UnitWalk {
+  const UnitTable* t;
+  int n_gemms, shares, total, bin, step;
+  int g, u, rounds;     // rounds: whole rounds left of GEMM g; -1: in the units behind them
+
+  __device__ __forceinline__ UnitWalk(const UnitTable* tab, int n, int shares_on, int total_units, int bin, int bins)
+      : t(tab), n_gemms(n), shares(shares_on), total(total_units), bin(bin), step(bins), g(shares_on ? -1 : 0),
+        u(bin - bins), rounds(-1) {}
+
+  // Move to the next unit; false when there is none.
+  __device__ __forceinline__ bool next() {
+    if (!shares) {
+      u += step;
+      return u < total;
+    }
+    for (;;) {
+      if (g >= 0) {
+        if (rounds > 0) {
+          --rounds;
+          u += step;
+          return true;
+        }
+        u = rounds == 0 ? t[g].lo : u + 1;
+        rounds = -1;
+        if (u < t[g].hi) return true;
+      }
+      if (++g >= n_gemms) return false;
+      rounds = t[g].rounds;
+      u = t[g].unit_begin + bin - step;
+    }
+  }
+  __device__ __forceinline__ bool last() const {
+    UnitWalk w = *this;
+    return !w.next();
+  }
+  __device__ __forceinline__ UnitCoord coord() const {
+    UnitCoord c;
+    int gi = g;
+    if (!shares)
+#pragma unroll 1
+      while (gi + 1 < n_gemms && u >= t[gi + 1].unit_begin) ++gi;
+    const UnitTable& w = t[gi];
+    const int local = u - w.unit_begin;
+    c.g = gi;
+    c.tile = local / w.split;
+    c.s = local - c.tile * w.split;
+    const int per_batch = w.tiles_m * w.tiles_n;
+    c.b = c.tile / per_batch;
+    const int t2 = c.tile - c.b * per_batch;
+    c.tm = t2 % w.tiles_m;
+    c.tn = t2 / w.tiles_m;
+    c.kb0 = (c.s * w.k_blocks) / w.split;
+    c.kb1 = ((c.s + 1) * w.k_blocks) / w.split;
+    return c;
+  }
+};
 
 __device__ __forceinline__ void trace_stamp(unsigned long long* trace, int slot) {
   if (trace) trace[blockIdx.x * kTracePerCta + slot] = ptx::global_timer();
@@ -510,6 +574,8 @@ __device__ __forceinline__ void send_chunk(const CView& w, const void* tmap_c, b
 // Store an accumulator tile of up to MMA_N columns (rows m0 .., columns n0 ..
 // n0 + ncols - 1 of C).  The next chunk's tensor-memory load is issued before
 // this chunk's barrier and store, so its latency is not on the chunk's chain.
+// (The load is unconditional, also past ncols: under a condition the compiler
+// kept every chunk's registers and spilled 2.7 KB a thread.)
 template <int MMA_N, bool OUT_BF16>
 __device__ __forceinline__ void store_tile(const CView& w, const void* tmap_c, bool tma, uint32_t staging,
                                            uint32_t& stg, uint32_t taddr, int et, int q, int m0, int n0, int ncols,
@@ -572,14 +638,55 @@ __device__ __forceinline__ void send_tile_wide(const CView& w, const void* tmap_
                              m0 + 32 * q, n0 + c0);
 }
 
-// Split-K, last split to arrive: sum the S partials of the tile in split order
-// 0, 1, ..., S-1 and store them.  `parts`: this lane's row of the
-// tile's first partial (layout [column / 4][row]), partial s `stride` float4
-// further on; the own split's values come from tensor memory.  Two splits'
-// partials are loaded before either is added, so their loads are in flight
-// together.  The sums leave through the staging buffers, the lanes along the
-// columns: for C whose rows are not 16-byte aligned (aligned rows are stored
-// from registers, which measured 3% faster on a set of split-K GEMMs).
+// Split-K, last split to arrive: columns c0 .. c0 + 31 of this lane's row,
+// summed over the S partials in split order 0, 1, ..., S-1.  `parts`: the row
+// in the tile's first partial (layout [column / 4][row]), partial s `stride`
+// float4 further on; the own split's values come from tensor memory.  Two
+// splits' partials are loaded before either is added, so their loads are in
+// flight together.
+__device__ __forceinline__ void sum_partials(const float4* parts, int stride, int S, int own_s, uint32_t taddr, int c0,
+                                             float (&v)[32]) {
+  uint32_t raw[32];
+  __syncwarp();
+  ptx::tmem_ld_32x32b_x32(taddr + c0, raw);
+  ptx::tmem_ld_wait();
+#pragma unroll
+  for (int j = 0; j < 32; ++j) v[j] = 0.0f;
+#pragma unroll 1
+  for (int s2 = 0; s2 < S; s2 += 2) {
+    const bool has_b = s2 + 1 < S;
+    float4 ta[8], tb[8];
+    const float4* pa = parts + size_t(s2) * stride + size_t(c0 / 4) * 128;
+#pragma unroll
+    for (int j4 = 0; j4 < 8; ++j4) {
+      const float4 own = make_float4(__uint_as_float(raw[4 * j4]), __uint_as_float(raw[4 * j4 + 1]),
+                                     __uint_as_float(raw[4 * j4 + 2]), __uint_as_float(raw[4 * j4 + 3]));
+      ta[j4] = (s2 == own_s) ? own : __ldcg(&pa[j4 * 128]);
+      tb[j4] = (!has_b || s2 + 1 == own_s) ? own : __ldcg(&pa[size_t(stride) + j4 * 128]);
+    }
+#pragma unroll
+    for (int j4 = 0; j4 < 8; ++j4) {
+      v[4 * j4] += ta[j4].x;
+      v[4 * j4 + 1] += ta[j4].y;
+      v[4 * j4 + 2] += ta[j4].z;
+      v[4 * j4 + 3] += ta[j4].w;
+    }
+    if (has_b) {
+#pragma unroll
+      for (int j4 = 0; j4 < 8; ++j4) {
+        v[4 * j4] += tb[j4].x;
+        v[4 * j4 + 1] += tb[j4].y;
+        v[4 * j4 + 2] += tb[j4].z;
+        v[4 * j4 + 3] += tb[j4].w;
+      }
+    }
+  }
+}
+
+// The same for a whole tile, leaving through the staging buffers with the
+// lanes along the columns: for C whose rows are not 16-byte aligned (aligned
+// rows are stored from registers, which measured 3% faster on a set of
+// split-K GEMMs).
 template <bool OUT_BF16>
 __device__ __forceinline__ void sum_and_store_tile(const CView& w, const float4* parts, int stride, int S, int own_s,
                                                    uint32_t staging, uint32_t& stg, uint32_t taddr, int et, int q,
@@ -591,43 +698,10 @@ __device__ __forceinline__ void sum_and_store_tile(const CView& w, const float4*
 #pragma unroll 1
     for (int h = 0; h < (OUT_BF16 ? 2 : 1) && live; ++h) {
       const int cc = c0 + 32 * h;
-      if (cc >= ncols) break;             // the chunk's second half lies past N (its columns are clipped)
-      uint32_t raw[32];
-      __syncwarp();
-      ptx::tmem_ld_32x32b_x32(taddr + cc, raw);
-      ptx::tmem_ld_wait();
+      if (cc >= ncols) break;             // the chunk's second half lies past N
       float v[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = 0.0f;
-#pragma unroll 1
-      for (int s2 = 0; s2 < S; s2 += 2) {
-        const bool has_b = s2 + 1 < S;
-        float4 ta[8], tb[8];
-        const float4* pa = parts + size_t(s2) * stride + size_t(cc / 4) * 128;
-#pragma unroll
-        for (int j4 = 0; j4 < 8; ++j4) {
-          const float4 own = make_float4(__uint_as_float(raw[4 * j4]), __uint_as_float(raw[4 * j4 + 1]),
-                                         __uint_as_float(raw[4 * j4 + 2]), __uint_as_float(raw[4 * j4 + 3]));
-          ta[j4] = (s2 == own_s) ? own : __ldcg(&pa[j4 * 128]);
-          tb[j4] = (!has_b || s2 + 1 == own_s) ? own : __ldcg(&pa[size_t(stride) + j4 * 128]);
-        }
-#pragma unroll
-        for (int j4 = 0; j4 < 8; ++j4) {
-          v[4 * j4] += ta[j4].x;
-          v[4 * j4 + 1] += ta[j4].y;
-          v[4 * j4 + 2] += ta[j4].z;
-          v[4 * j4 + 3] += ta[j4].w;
-        }
-        if (has_b) {
-#pragma unroll
-          for (int j4 = 0; j4 < 8; ++j4) {
-            v[4 * j4] += tb[j4].x;
-            v[4 * j4 + 1] += tb[j4].y;
-            v[4 * j4 + 2] += tb[j4].z;
-            v[4 * j4 + 3] += tb[j4].w;
-          }
-        }
-      }
+      sum_partials(parts, stride, S, own_s, taddr, cc, v);
+      uint32_t raw[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) raw[j] = __float_as_uint(v[j]);
       stage_cols<OUT_BF16>(buf + uint32_t(q) * kWarpChunk, et & 31, h, raw);
@@ -792,17 +866,12 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
   uint64_t* drain = bars + 2 * STAGES + 2 * ACC;
   uint64_t* redbar = drain + 1;        // cluster split-K: 2 barriers, alternating by unit
   uint64_t* recvbar = redbar + 2;      // pushed cluster reduction: bytes received
-  uint64_t* ufull = recvbar + 1;       // unit ring: the producer published the unit index
-  uint64_t* uempty = ufull + kUnitRing;  // unit ring: the MMA thread and the epilogue read it
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(uempty + kUnitRing);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(recvbar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* last_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
   volatile int* units_taken = reinterpret_cast<volatile int*>(tmem_slot + 3);
   UnitTable* utab = reinterpret_cast<UnitTable*>(tmem_slot + 4);   // MAXG entries, inside the 1 KB barrier area
-  volatile int* uring = reinterpret_cast<volatile int*>(utab + MAXG);   // kUnitRing unit indices
-  static_assert((2 * STAGES + 2 * ACC + 4 + 2 * kUnitRing) * 8 + 16 + MAXG * int(sizeof(UnitTable)) +
-                        kUnitRing * 4 <= 1024,
-                "barrier area");
+  static_assert((2 * STAGES + 2 * ACC + 4) * 8 + 16 + MAXG * int(sizeof(UnitTable)) <= 1024, "barrier area");
   const int n_gemms = p.n_gemms;
 
   const uint32_t tiles_base = ptx::smem_u32(smem);
@@ -811,7 +880,7 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
   unsigned long long* const trace = p.trace;
   // the next launch on this stream may start its set-up now; it waits
   // (griddep_wait) for this grid to complete before touching global memory
-  ptx::griddep_launch_dependents();
+  if (!p.late_trigger) ptx::griddep_launch_dependents();
 
   // pushed cluster reduction: one unit per CTA, every GEMM split S = cluster
   const bool push_on = kPush && p.cluster > 0 && p.total_units == int(gridDim.x);
@@ -845,10 +914,6 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
       ptx::mbar_init(ptx::smem_u32(&redbar[1]), uint32_t(p.cluster));
     }
     if (push_on) ptx::mbar_init(ptx::smem_u32(recvbar), 1);
-    for (int q = 0; q < kUnitRing; ++q) {
-      ptx::mbar_init(ptx::smem_u32(&ufull[q]), 1);
-      ptx::mbar_init(ptx::smem_u32(&uempty[q]), 2);
-    }
     *abort_flag = 0;
     *last_flag = 0;
     *units_taken = 0;
@@ -864,16 +929,7 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), TMEM_COLS);
     ptx::tmem_relinquish();
   } else if (warp == 2) {
-    for (int g = lane; g < p.n_gemms; g += 32) {
-      UnitTable e;
-      e.unit_begin = p.g[g].unit_begin;
-      e.split = p.g[g].split;
-      e.tiles_m = p.g[g].tiles_m;
-      e.tiles_n = p.g[g].tiles_n;
-      e.k_blocks = p.g[g].k_blocks;
-      e.n = p.g[g].n;
-      utab[g] = e;
-    }
+    fill_unit_table(utab, p, int(blockIdx.x), lane);
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -883,22 +939,20 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
   if (p.cluster > 0) ptx::cluster_sync_all();
   const uint32_t tmem_base = *tmem_slot;
   const uint64_t wlim = p.wait_ns ? p.wait_ns : ptx::kWaitLimitNs;
+  UnitWalk walk(utab, n_gemms, p.shares.on, p.total_units, int(blockIdx.x), int(gridDim.x));
   if (threadIdx.x == 0) trace_stamp(trace, kTrPreWait);
   // set-up above touched only shared and tensor memory; global memory (the
   // operands, C, the split-K workspace) only after the previous grid is done.
   // Early mode: the producer (reading A and B only, asserted not written by
   // an earlier kernel) and the MMA thread (shared and tensor memory only)
   // go ahead; the epilogue, which writes C and the workspace, still waits.
-  // A launch that hands units out from a workspace counter loads its first
-  // unit (this CTA's own) early too; the producer waits before its first
-  // read of the counter, which the previous launch over the same GEMMs
-  // zeroes as it ends.
   const bool early = p.early_loads != 0 && warp < 2;
   // In early mode the epilogue waits where it first writes global memory
   // (below): a CTA's last tile is read out of tensor memory into the idle
   // operand ring before that wait, so only its stores are left after it.
   const bool epi_defer = p.early_loads != 0 && warp >= 2;
   if (!early && !epi_defer) ptx::griddep_wait();
+  if (p.late_trigger) ptx::griddep_launch_dependents();
   if (threadIdx.x == 64 && !epi_defer) trace_stamp(trace, kTrSetup);   // the first epilogue thread waits
 
   if (warp == 0) {
@@ -907,31 +961,11 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
       int stage = 0;
       uint32_t phase = 0, issued = 0, last_phase = 0;
       bool ok = true, stalled = false;
-      int u = blockIdx.x, taken = 0;
-      for (int seq = 0; ok && !stalled; ++seq) {
-        if (p.dyn) {
-          // publish the unit (or the end: an index past the last unit) to
-          // the MMA thread and the epilogue
-          const int slot = seq % kUnitRing;
-          if (seq >= kUnitRing &&
-              !ptx::mbar_wait(ptx::smem_u32(&uempty[slot]), uint32_t((seq / kUnitRing) - 1) & 1u, abort_flag,
-                              wlim)) {
-            ok = false;
-            break;
-          }
-          uring[slot] = u;
-          ptx::mbar_arrive(ptx::smem_u32(&ufull[slot]));
-        }
-        if (u >= p.total_units) break;
+      int taken = 0;
+      while (ok && !stalled && walk.next()) {
         ++taken;
-        // the next unit, taken now so that the counter's latency overlaps
-        // this unit's loads — except after an early start, where the counter
-        // is read once the first unit's loads are out and the previous grid
-        // is done
-        const bool defer_next = p.dyn && early && seq == 0;
-        int next = defer_next ? 0 : (p.dyn ? int(gridDim.x + atomicAdd(p.dyn, 1u)) : u + int(gridDim.x));
         if (issued == 0) trace_stamp(trace, kTrProducerGo);
-        const UnitCoord c = decode_unit_tab(utab, n_gemms, u);
+        const UnitCoord c = walk.coord();
         const void* ta = &p.tmap_a[c.g];
         const void* tb = &p.tmap_b[c.g];
         const int m0 = c.tm * TILE_M;
@@ -977,12 +1011,6 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
             phase ^= 1;
           }
         }
-        if (defer_next) {
-          if (!ok || stalled) break;
-          ptx::griddep_wait();
-          next = int(gridDim.x + atomicAdd(p.dyn, 1u));
-        }
-        u = next;
       }
       *units_taken = taken;
       if (!ok) {
@@ -998,19 +1026,9 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, acc_used = 0;
       bool ok = true, any = false;
-      for (int seq = 0; ok; ++seq) {
-        int u = int(blockIdx.x) + seq * int(gridDim.x);   // static round-robin
-        if (p.dyn) {
-          const int slot = seq % kUnitRing;
-          if (!ptx::mbar_wait(ptx::smem_u32(&ufull[slot]), uint32_t(seq / kUnitRing) & 1u, abort_flag, wlim)) {
-            ok = false;
-            break;
-          }
-          u = uring[slot];
-          ptx::mbar_arrive(ptx::smem_u32(&uempty[slot]));
-        }
-        if (u >= p.total_units) break;
-        const UnitCoord c = decode_unit_tab(utab, n_gemms, u);
+      bool first = true;
+      while (ok && walk.next()) {
+        const UnitCoord c = walk.coord();
         // an accumulator is waited for only once it has been used before
         if ((acc_used >> acc & 1) &&
             !ptx::mbar_wait(ptx::smem_u32(&tempty[acc]), acc_phase ^ 1, abort_flag, wlim)) {
@@ -1050,7 +1068,8 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
         }
         if (!ok) break;
         ptx::mma_commit(ptx::smem_u32(&tfull[acc]));        // accumulator complete
-        if (seq == 0) trace_stamp(trace, kTrFirstMmaDone);
+        if (first) trace_stamp(trace, kTrFirstMmaDone);
+        first = false;
         if (++acc == ACC) {
           acc = 0;
           acc_phase ^= 1;
@@ -1081,20 +1100,9 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
       waited = true;
       if (et == 0) trace_stamp(trace, kTrSetup);
     };
-    for (int seq = 0;; ++seq) {
-      const int slot = seq % kUnitRing;
-      int u = int(blockIdx.x) + seq * int(gridDim.x);     // static round-robin
-      if (p.dyn) {
-        bool okq = ptx::mbar_wait(ptx::smem_u32(&ufull[slot]), uint32_t(seq / kUnitRing) & 1u, abort_flag, wlim);
-        okq = ptx::named_bar_and(1, 128, okq);
-        if (!okq) {
-          if (et == 0) raise_error(p.err, abort_flag, kErrEpilogueWait);
-          break;
-        }
-        u = uring[slot];
-      }
-      if (u >= p.total_units) break;
-      const UnitCoord c = decode_unit_tab(utab, n_gemms, u);
+    bool first_unit = true;
+    for (; walk.next(); first_unit = false) {
+      const UnitCoord c = walk.coord();
       // the GEMM's output description, read from the parameter block while
       // the accumulator is still being computed
       const GemmWork w = p.g[c.g];
@@ -1106,10 +1114,7 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
         if (et == 0) raise_error(p.err, abort_flag, kErrEpilogueWait);
         break;
       }
-      // every epilogue thread has read the unit's slot (the barrier above)
-      if (p.dyn && et == 0) ptx::mbar_arrive(ptx::smem_u32(&uempty[slot]));
       ptx::tc_fence_after();
-      const bool first_unit = (seq == 0);
       if (first_unit && et == 0) trace_stamp(trace, kTrFirstAcc);
       const int m0 = c.tm * TILE_M;
       const int n0 = c.tn * TILE_N;
@@ -1120,7 +1125,7 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
       // holds the tile: they keep no staging buffers and store their other
       // tiles directly)
       static_assert(!EPI_TMA || kWideFits, "the ring holds a whole tile");
-      const bool wide = kWideFits && w.split == 1 && p.dyn == nullptr && u + int(gridDim.x) >= p.total_units;
+      const bool wide = kWideFits && w.split == 1 && walk.last();
       const int ncols = min(MMA_N, w.n - n0);
       // the cluster reductions on chip exchange partials through shared
       // memory only and wait just before their stores
@@ -1315,46 +1320,8 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
                                          staging, stg, taddr, et, q, m0, n0, ncols);
 #pragma unroll 1
           for (int c0 = 0; c0 < (staged ? 0 : MMA_N); c0 += 32) {
-            uint32_t raw[32];
-            __syncwarp();
-            ptx::tmem_ld_32x32b_x32(taddr + c0, raw);
-            ptx::tmem_ld_wait();
             float v[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = 0.0f;
-            // two splits' partials are loaded before either is added, so their
-            // loads are in flight together; the sum runs in split order
-            // 0, 1, ..., S-1 (the own split's values come from tensor memory)
-#pragma unroll 1
-            for (int s2 = 0; s2 < w.split; s2 += 2) {
-              const bool has_b = s2 + 1 < w.split;
-              float4 ta[8], tb[8];
-              const float4* pa = part_base + size_t(c.tile * w.split + s2) * TILE_F4;
-              const float4* pb = part_base + size_t(c.tile * w.split + s2 + 1) * TILE_F4;
-#pragma unroll
-              for (int j4 = 0; j4 < 8; ++j4) {
-                const float4 own = make_float4(__uint_as_float(raw[4 * j4]), __uint_as_float(raw[4 * j4 + 1]),
-                                               __uint_as_float(raw[4 * j4 + 2]), __uint_as_float(raw[4 * j4 + 3]));
-                ta[j4] = (s2 == c.s) ? own : __ldcg(&pa[((c0 / 4) + j4) * 128 + r]);
-                tb[j4] = (!has_b || s2 + 1 == c.s) ? own : __ldcg(&pb[((c0 / 4) + j4) * 128 + r]);
-              }
-#pragma unroll
-              for (int j4 = 0; j4 < 8; ++j4) {
-                v[4 * j4] += ta[j4].x;
-                v[4 * j4 + 1] += ta[j4].y;
-                v[4 * j4 + 2] += ta[j4].z;
-                v[4 * j4 + 3] += ta[j4].w;
-              }
-              if (has_b) {
-#pragma unroll
-                for (int j4 = 0; j4 < 8; ++j4) {
-                  v[4 * j4] += tb[j4].x;
-                  v[4 * j4 + 1] += tb[j4].y;
-                  v[4 * j4 + 2] += tb[j4].z;
-                  v[4 * j4 + 3] += tb[j4].w;
-                }
-              }
-            }
+            sum_partials(part_base + size_t(c.tile * w.split) * TILE_F4 + r, TILE_F4, w.split, c.s, taddr, c0, v);
             store_chunk<SWAP, OUT_BF16>(cv, m0, n0, r, c0, v);
           }
           if (et == 0) w.ws_cnt[c.tile] = 0u;     // leave the counter zeroed for the next run
@@ -1380,16 +1347,6 @@ __global__ void __launch_bounds__(192, MIN_CTAS) go_gemm_kernel(const __grid_con
   if (threadIdx.x == 0) {
     trace_stamp(trace, kTrEnd);
     if (trace) trace[blockIdx.x * kTracePerCta + kTrUnits] = *units_taken;
-    if (p.dyn) {
-      // every CTA has stopped taking units once all have counted themselves
-      // out: the last one zeroes the counters for the next launch
-      __threadfence();
-      if (atomicAdd(p.dyn + 1, 1u) == gridDim.x - 1) {
-        p.dyn[0] = 0u;
-        p.dyn[1] = 0u;
-        __threadfence();
-      }
-    }
   }
   // no CTA of a cluster leaves while a peer may still signal its barriers
   // (every role's waits are bounded, so every CTA gets here)

@@ -15,12 +15,13 @@
 // jointly with the peer and, in the even CTA, issues the MMAs and commits
 // (multicast to both CTAs' barriers), warps 2-5 drain the CTA's own half of
 // the accumulator.  Units (256 x 256 tiles, or with a K split S, S K-ranges
-// of a tile) go to pairs round-robin; both CTAs of a pair walk the same
-// sequence.  With S > 1 each CTA publishes its 128 x 256 fp32 partial to the
-// workspace and the last split to arrive for a tile half sums the S partials
-// in split order and stores C.  Every wait is bounded; before leaving,
-// each CTA waits (bounded) until every arrival the peer owes its barriers has
-// landed, then the pair meets at a cluster barrier.
+// of a tile) go to pairs round-robin, or in shares over several GEMMs (see
+// UnitShares); both CTAs of a pair walk the same sequence.  With S > 1 each
+// CTA publishes its 128 x 256 fp32 partial to the workspace and the last split
+// to arrive for a tile half sums the S partials in split order and stores C.
+// Every wait is bounded; before leaving, each CTA waits (bounded) until every
+// arrival the peer owes its barriers has landed, then the pair meets at a
+// cluster barrier.
 #pragma once
 
 #include "go_kernel.cuh"
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
   const int pair = blockIdx.x >> 1;
   const int n_pairs = gridDim.x >> 1;
   unsigned long long* const trace = p.trace;
-  ptx::griddep_launch_dependents();   // see go_gemm_kernel
+  if (!p.late_trigger) ptx::griddep_launch_dependents();   // see go_gemm_kernel
 
   if (threadIdx.x == 0) {
     trace_stamp(trace, kTrStart);
@@ -100,16 +101,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
     ptx::tmem_alloc_pair(ptx::smem_u32(tmem_slot), TMEM_COLS);
     ptx::tmem_relinquish_pair();
   } else if (warp == 2) {
-    for (int g = lane; g < p.n_gemms; g += 32) {
-      UnitTable e;
-      e.unit_begin = p.g[g].unit_begin;
-      e.split = p.g[g].split;
-      e.tiles_m = p.g[g].tiles_m;
-      e.tiles_n = p.g[g].tiles_n;
-      e.k_blocks = p.g[g].k_blocks;
-      e.n = p.g[g].n;
-      utab[g] = e;
-    }
+    fill_unit_table(utab, p, pair, lane);
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -118,6 +110,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const uint64_t wlim = p.wait_ns ? p.wait_ns : ptx::kWaitLimitNs;
+  UnitWalk walk(utab, n_gemms, p.shares.on, p.total_units, pair, n_pairs);
   // global memory only after the previous grid is done; in early mode the
   // load and MMA roles go ahead (see go_gemm_kernel) and the epilogue waits
   const bool early = p.early_loads != 0 && warp < 2;
@@ -125,6 +118,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
   // (below); a CTA's last tile is staged in the idle ring before that wait
   const bool epi_defer = p.early_loads != 0 && warp >= 2;
   if (!early && !epi_defer) ptx::griddep_wait();
+  if (p.late_trigger) ptx::griddep_launch_dependents();
   if (threadIdx.x == 64 && !epi_defer) trace_stamp(trace, kTrSetup);   // the first epilogue thread waits
 
   if (warp == 0) {
@@ -133,8 +127,8 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
       int stage = 0;
       uint32_t phase = 0, issued = 0, last_phase = 0;
       bool ok = true;
-      for (int u = pair; ok && u < p.total_units; u += n_pairs) {
-        const UnitCoord c = decode_unit_tab(utab, n_gemms, u);
+      while (ok && walk.next()) {
+        const UnitCoord c = walk.coord();
         const void* ta = &p.tmap_a[c.g];
         const void* tb = &p.tmap_b[c.g];
         const int m0 = c.tm * 256 + int(rank) * 128;
@@ -187,9 +181,9 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
       // ------------------------------------------------- MMA issuer (even CTA)
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, acc_used = 0;
-      bool ok = true, any = false;
-      for (int u = pair; ok && u < p.total_units; u += n_pairs) {
-        const UnitCoord c = decode_unit_tab(utab, n_gemms, u);
+      bool ok = true, any = false, first = true;
+      while (ok && walk.next()) {
+        const UnitCoord c = walk.coord();
         // both CTAs drained this accumulator (the odd CTA signals with a
         // cluster-scope release, so wait with a cluster-scope acquire); the
         // first use of an accumulator needs no wait
@@ -226,7 +220,8 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
         }
         if (!ok) break;
         ptx::mma_commit_pair_multicast(ptx::smem_u32(&tfull[acc]), 0x3);
-        if (u == pair) trace_stamp(trace, kTrFirstMmaDone);
+        if (first) trace_stamp(trace, kTrFirstMmaDone);
+        first = false;
         if (++acc == ACC) {
           acc = 0;
           acc_phase ^= 1;
@@ -256,8 +251,9 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
       waited = true;
       if (et == 0) trace_stamp(trace, kTrSetup);
     };
-    for (int u = pair; u < p.total_units; u += n_pairs) {
-      const UnitCoord c = decode_unit_tab(utab, n_gemms, u);
+    bool first_unit = true;
+    for (; walk.next(); first_unit = false) {
+      const UnitCoord c = walk.coord();
       const GemmWork w = p.g[c.g];                 // read while the accumulator is computed
       const CView cv = c_view<OUT_BF16>(w, c.b);
       bool ok = ptx::mbar_wait(ptx::smem_u32(&tfull[acc]), acc_phase, abort_flag, wlim);
@@ -267,7 +263,6 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
         break;
       }
       ptx::tc_fence_after();
-      const bool first_unit = (u == pair);
       if (first_unit && et == 0) trace_stamp(trace, kTrFirstAcc);
       const int m0 = c.tm * 256 + int(rank) * 128;
       const int n0 = c.tn * 256;
@@ -276,7 +271,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
       // ready) and no load is left, so the operand ring is idle and stages
       // the whole tile (128 KB fp32 / 64 KB bf16 of its 192 KB) before the
       // wait; only the stores follow it
-      const bool wide = w.split == 1 && u + n_pairs >= p.total_units;
+      const bool wide = w.split == 1 && walk.last();
       static_assert(STAGES * STAGE_BYTES >= 256 * 512, "the ring holds a whole tile half");
       const int ncols = min(256, w.n - n0);
       const bool tma = w.c_tma != 0;
@@ -328,29 +323,8 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
                                          ncols);
 #pragma unroll 1
           for (int c0 = 0; c0 < (staged ? 0 : nc); c0 += 32) {
-            uint32_t raw[32];
-            __syncwarp();
-            ptx::tmem_ld_32x32b_x32(taddr + c0, raw);
-            ptx::tmem_ld_wait();
             float v[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = 0.0f;
-#pragma unroll 1
-            for (int s2 = 0; s2 < w.split; ++s2) {
-              float4 t[8];
-#pragma unroll
-              for (int j4 = 0; j4 < 8; ++j4)
-                t[j4] = (s2 == c.s) ? make_float4(__uint_as_float(raw[4 * j4]), __uint_as_float(raw[4 * j4 + 1]),
-                                                   __uint_as_float(raw[4 * j4 + 2]), __uint_as_float(raw[4 * j4 + 3]))
-                                    : __ldcg(&parts[size_t(s2) * TILE_F4 + ((c0 / 4) + j4) * 128 + r]);
-#pragma unroll
-              for (int j4 = 0; j4 < 8; ++j4) {
-                v[4 * j4] += t[j4].x;
-                v[4 * j4 + 1] += t[j4].y;
-                v[4 * j4 + 2] += t[j4].z;
-                v[4 * j4 + 3] += t[j4].w;
-              }
-            }
+            sum_partials(parts + r, TILE_F4, w.split, c.s, taddr, c0, v);
             store_chunk<false, OUT_BF16>(cv, m0, n0, r, c0, v);
           }
           if (et == 0) w.ws_cnt[half] = 0u;     // leave the counter zeroed for the next run
@@ -381,7 +355,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
     trace_stamp(trace, kTrEnd);
     if (trace) {
       int n = 0;
-      for (int u = pair; u < p.total_units; u += n_pairs) ++n;
+      for (UnitWalk all(utab, n_gemms, p.shares.on, p.total_units, pair, n_pairs); all.next();) ++n;
       trace[blockIdx.x * kTracePerCta + kTrUnits] = n;
     }
   }

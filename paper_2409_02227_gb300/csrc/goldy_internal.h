@@ -122,9 +122,6 @@ struct GemmPlan {
   size_t ws_part_off = 0;   // byte offsets into the caller's workspace
   size_t ws_cnt_off = 0;
   size_t ws_bytes = 0;
-  // a fused launch led by this GEMM may hand out its units through a pair of
-  // counters here (fused schedules of several GEMMs; kNoOffset otherwise)
-  size_t ws_dyn_off = ~size_t(0);
 };
 
 struct Group {
@@ -149,6 +146,13 @@ const void* kernel_fn_k7(int out_bf16, int fused);
 const void* kernel_fn_k8(int out_bf16, int fused);
 const void* kernel_fn_k9(int out_bf16, int fused);
 const void* kernel_fn_k10(int out_bf16, int fused);
+// The kernel over GEMMs of different single-CTA tile shapes, and its dynamic
+// shared memory: a 192 KB operand ring, two 16 KB staging buffers, 1 KB for
+// alignment, 1 KB for barriers.
+const void* kernel_fn_set(int out_bf16);
+constexpr int kSetRing = 4 * 49152;
+constexpr int kSetSmemBytes = kSetRing + 2 * 16384 + 2048;
+constexpr int kSetMaxStages = 8;
 
 // Element-wise add (ewise.cu): Z = X + Y over n elements.
 struct EwiseParams {
@@ -167,6 +171,7 @@ const void* ewise_kernel_fn(int bf16);
 
 struct goldy_schedule {
   int flags = 0;
+  bool auto_plan = false;   // planned by GOLDY_PLAN_AUTO (fused: one launch per kernel family, see run_impl)
   int max_streams = 1;
   size_t workspace_bytes = 0;
   std::vector<goldy::GemmPlan> gemms;
@@ -193,6 +198,13 @@ goldy_status ok();
 goldy_status check_desc(const goldy_gemm_desc& d, int index);
 // fill derived fields and workspace offsets (planner.cpp)
 void finalize_schedule(goldy_schedule* s);
+// Deal out the units of n GEMMs (units[g] of cost[g] each; most costly GEMM
+// first) to `bins` bins in equal shares: of GEMM g, bin b gets units b,
+// b + bins, ... below rounds[g] * bins, and units first[g * (bins + 1) + b] ..
+// first[g * (bins + 1) + b + 1] - 1; rounds[g] is 0 unless rotate[g]
+// (planner.cpp).
+void assign_units(int n, const int64_t* units, const double* cost, const bool* rotate, int bins, int32_t* rounds,
+                  int32_t* first);
 // release CUDA-side state (runtime.cu; no-op without it)
 void runtime_release(Runtime* rt);
 }  // namespace goldy

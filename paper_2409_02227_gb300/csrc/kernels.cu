@@ -1,9 +1,11 @@
 // Instantiates the GO-Kernel template for one kind (compile with
-// -DGOLDY_KIND=k, k in 0 .. kNumKinds-1), both output dtypes, and both launch
+// -DGOLDY_KIND=k, k in 0 .. kNumKinds-1; k = kNumKinds: the kernel that mixes
+// them), both output dtypes, and both launch
 // forms (one GEMM per launch, or up to kMaxFused GEMMs).  One object per kind
 // keeps the build parallel.
 #include "go_kernel.cuh"
 #include "go_kernel_pair.cuh"
+#include "go_kernel_set.cuh"
 #include "goldy_internal.h"
 
 #ifndef GOLDY_KIND
@@ -15,6 +17,14 @@
 
 namespace goldy {
 
+#if GOLDY_KIND == 11
+// The kernel over GEMMs of different tile shapes (always the fused form).
+static_assert(kSetRingBytes + 2 * 16384 + 2048 == kSetSmemBytes, "host and kernel agree on the shared memory");
+const void* kernel_fn_set(int out_bf16) {
+  return out_bf16 ? reinterpret_cast<const void*>(&go_gemm_set_kernel<true, kMaxFused>)
+                  : reinterpret_cast<const void*>(&go_gemm_set_kernel<false, kMaxFused>);
+}
+#else
 // Inside a template, `if constexpr` discards the other family entirely.
 template <int KIND>
 const void* select_kernel(int out_bf16, int fused) {
@@ -48,5 +58,6 @@ const void* select_kernel(int out_bf16, int fused) {
 const void* GOLDY_CAT(kernel_fn_k, GOLDY_KIND)(int out_bf16, int fused) {
   return select_kernel<GOLDY_KIND>(out_bf16, fused);
 }
+#endif
 
 }  // namespace goldy

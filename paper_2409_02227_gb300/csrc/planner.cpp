@@ -25,8 +25,10 @@
 #include <cstring>
 #include <fstream>
 #include <iterator>
+#include <limits>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "goldy_internal.h"
@@ -374,15 +376,64 @@ void finalize_schedule(goldy_schedule* s) {
       gp.ws_bytes = off - gp.ws_part_off;
     }
   }
-  // fused schedules of several GEMMs: a pair of unit counters per GEMM (a
-  // fused launch uses its first member's); zero like the split-K counters
-  if ((s->flags & GOLDY_PLAN_FUSED) && s->gemms.size() > 1) {
-    for (size_t i = 0; i < s->gemms.size(); ++i) s->gemms[i].ws_dyn_off = off + 8 * i;
-    off = align(off + 8 * s->gemms.size());
-  } else {
-    for (auto& gp : s->gemms) gp.ws_dyn_off = ~size_t(0);
-  }
+  // fused schedules of several GEMMs keep 8 bytes per GEMM at the end of the
+  // workspace, reserved (part of the size goldy_schedule_query documents)
+  if ((s->flags & GOLDY_PLAN_FUSED) && s->gemms.size() > 1) off = align(off + 8 * s->gemms.size());
   s->workspace_bytes = off;
+}
+
+// Longest-processing-time order with whole GEMMs' units at a time: the bins
+// are filled like a vessel, each GEMM's units raising the lowest bins to a
+// common level as far as whole units allow, the rest one each to the lowest.
+// A microsecond or two per GEMM.
+void assign_units(int n, const int64_t* units, const double* cost, const bool* rotate, int bins, int32_t* rounds,
+                  int32_t* first) {
+  std::vector<double> load(size_t(bins), 0.0);
+  std::vector<int64_t> take(static_cast<size_t>(bins));
+  std::vector<std::pair<double, int>> low(static_cast<size_t>(bins));
+  for (int g = 0; g < n; ++g) {
+    const double c = std::max(cost[g], 1e-9), work = double(units[g]) * c;
+    // the level at which the bins below it would hold all units, if units
+    // could be cut: bins above the level of all bins only lower it
+    double level = std::numeric_limits<double>::infinity();
+    for (;;) {
+      double sum = work;
+      int below = 0;
+      for (double l : load)
+        if (l < level) {
+          sum += l;
+          ++below;
+        }
+      const double next = sum / double(std::max(below, 1));
+      if (!(next < level)) break;
+      level = next;
+    }
+    int64_t left = units[g];
+    for (int b = 0; b < bins; ++b) {
+      const double room = (level - load[size_t(b)]) / c;
+      take[size_t(b)] = room > 0.0 ? std::min<int64_t>(left, int64_t(room + 1e-9)) : 0;
+      left -= take[size_t(b)];
+      low[size_t(b)] = {load[size_t(b)] + c * double(take[size_t(b)]), b};
+    }
+    while (left > 0) {
+      const size_t m = size_t(std::min<int64_t>(left, bins));
+      std::nth_element(low.begin(), low.begin() + (m - 1), low.end());   // equal loads: the smaller bin first
+      for (size_t k = 0; k < m; ++k) {
+        ++take[size_t(low[k].second)];
+        low[k].first += c;
+      }
+      left -= int64_t(m);
+    }
+    for (const auto& x : low) load[size_t(x.second)] = x.first;
+    const int64_t whole = rotate[g] ? *std::min_element(take.begin(), take.end()) : 0;
+    rounds[g] = int32_t(whole);
+    int32_t at = int32_t(whole) * bins;
+    for (int b = 0; b < bins; ++b) {
+      first[g * (bins + 1) + b] = at;
+      at += int32_t(take[size_t(b)] - whole);
+    }
+    first[g * (bins + 1) + bins] = at;
+  }
 }
 
 }  // namespace goldy
@@ -560,7 +611,8 @@ extern "C" goldy_status goldy_plan_ex(const goldy_gemm_desc* descs, int n, const
       s->gemms[i].slot = int(j % size_t(groups[g].cd));
     }
   }
-  if (policy == GOLDY_PLAN_AUTO) one_kind_per_wave(s);
+  s->auto_plan = policy == GOLDY_PLAN_AUTO;
+  if (s->auto_plan) one_kind_per_wave(s);
   finalize_schedule(s);
   *out = s;
   return ok();

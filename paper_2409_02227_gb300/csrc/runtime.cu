@@ -83,6 +83,7 @@ thread_local bool t_pdl = true;
 // early operand loads, the bounded-wait limit, and the test stall hook
 // (first launch of the run only).
 thread_local int32_t t_early = 0;
+thread_local int32_t t_late = 0;    // LaunchParams::late_trigger of the next launch
 thread_local uint64_t t_wait_ns = 0;
 thread_local int32_t t_stall = 0;
 // Launch priority of the next GO-Kernel launch (kNoPriority: the stream's).
@@ -104,6 +105,7 @@ struct DeviceState {
   int prio_least = 0, prio_greatest = 0;    // cudaDeviceGetStreamPriorityRange
   int* err_word = nullptr;
   int ctas_per_sm[kNumKinds][2][2] = {};   // [kind][bf16 out][fused]; 0 = not yet set up
+  bool set_ready[2] = {};                  // the mixed-shape kernel, set up per output dtype
   int cluster_ok[kNumKinds][2][2][4] = {};  // [..][log2 cluster size]; 0 unknown, 1 yes, -1 no
 };
 
@@ -182,6 +184,17 @@ goldy_status kernel_setup(DeviceState& d, int kind, int out_bf16, int fused, int
     c = occ;
   }
   *ctas = c;
+  return GOLDY_OK;
+}
+
+// The same for the kernel over GEMMs of different tile shapes (one CTA per SM).
+goldy_status set_kernel_setup(DeviceState& d, int out_bf16) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (d.set_ready[out_bf16]) return GOLDY_OK;
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel_fn_set(out_bf16), cudaFuncAttributeMaxDynamicSharedMemorySize, kSetSmemBytes);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+  d.set_ready[out_bf16] = true;
   return GOLDY_OK;
 }
 
@@ -406,6 +419,8 @@ goldy_status fill_slot(LaunchParams<MAXG>& p, int j, const GemmPlan& gp, const v
   w.split = gp.split;
   w.k_blocks = int32_t(gp.k_blocks);
   w.unit_begin = unit_begin;
+  w.mma_n = k.mma_n;
+  w.swap = k.swap_ab;
   // C through TMA stores: kinds that keep staging buffers, 16-byte aligned C
   // and rows; the epilogue writes 128-byte rows (32 fp32 / 64 bf16 columns)
   const size_t es = g.c_dtype == GOLDY_BF16 ? 2 : 4;
@@ -577,6 +592,7 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
   p.err = d.err_word;
   p.wait_ns = t_wait_ns;
   p.early_loads = t_early;
+  p.late_trigger = t_late;
   p.stall_test = t_stall;
   t_stall = 0;
 
@@ -601,55 +617,106 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
   return GOLDY_OK;
 }
 
-// One launch over the tiles of `count` (<= kMaxFused) GEMMs of one kind and
-// output dtype.  The grid cap is the sum of the members' own caps (each
-// GO-Kernel keeps the share of the GPU it was tuned for), at most the whole
-// GPU.
-goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* members_in, int count,
-                          const void* const* A, const void* const* B, void* const* C, uint8_t* ws,
+// What one unit of a GEMM costs a CTA (pair), in nanoseconds, for dealing out
+// the units of a launch in equal shares: the slower of its main loop and of
+// writing its tile, plus a fixed part.  The rates are those of a GPU busy with
+// such units: per K block a 256-wide pair tile takes 270 ns of tensor core
+// time (half that for 128 columns), a single CTA's operands arrive at about 85
+// bytes/ns, a tile leaves at about 45 bytes/ns (each SM's share of the memory
+// rate).  Only the ratios matter.
+double unit_cost(const GemmPlan& gp) {
+  const KindInfo& k = kKinds[gp.kind];
+  const goldy_gemm_desc& g = gp.desc;
+  const double rows = double(g.M) / double(gp.tiles_m), cols = double(g.N) / double(gp.tiles_n);
+  const double kb = double(gp.k_blocks) / double(gp.split);
+  const double es = gp.split > 1 ? 4.0 : g.c_dtype == GOLDY_BF16 ? 2.0 : 4.0;
+  double per_kb, out = rows * cols * es / 45.0;
+  if (k.pair) {
+    per_kb = g.N <= 128 ? 140.0 : 270.0;
+    out *= 0.5;
+  } else {
+    per_kb = std::max(270.0 * k.mma_n / 256.0, (rows + cols) * 128.0 / 85.0);
+  }
+  return std::max(kb * per_kb, out) + 500.0;
+}
+
+// Equal shares of a launch's units for its `bins` CTAs (pairs); `members`
+// sorted by descending unit cost.  Left off (round-robin) when the table
+// cannot hold them.
+void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* members, int count, int bins) {
+  sh.on = 0;
+  if (count < 2 || bins > kMaxBins) return;
+  int64_t units[kMaxFused];
+  double cost[kMaxFused];
+  bool rotate[kMaxFused];
+  for (int j = 0; j < count; ++j) {
+    units[j] = s->gemms[members[j]].units;
+    // a split tile's K ranges are neighbouring units: one bin takes them one
+    // after another, so that few partials wait for the rest (a set of split-K
+    // GEMMs: 45.6 -> 40.3 us)
+    rotate[j] = s->gemms[members[j]].split == 1;
+    cost[j] = unit_cost(s->gemms[members[j]]);
+    if (units[j] > 65535) return;
+  }
+  static thread_local int32_t first[kMaxFused * (kMaxBins + 1)];
+  int32_t rounds[kMaxFused];
+  assign_units(count, units, cost, rotate, bins, rounds, first);
+  for (int j = 0; j < count; ++j) sh.rounds[j] = uint16_t(rounds[j]);
+  for (int j = 0; j < count; ++j)
+    for (int b = 0; b <= bins; ++b) sh.first[j][b] = uint16_t(first[j * (bins + 1) + b]);
+  sh.on = 1;
+}
+
+// One launch over the tiles of `count` (<= kMaxFused) GEMMs of one output
+// dtype: of one kind, or (`mixed`) of any single-CTA kinds through the kernel
+// that reads the tile shape per GEMM.  The grid cap is the sum of the members'
+// own caps (each GO-Kernel keeps the share of the GPU it was tuned for), at
+// most the whole GPU; `whole`: the whole GPU (a launch that carries several
+// waves of a run, or several kinds).
+goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* members_in, int count, bool mixed,
+                          bool whole, const void* const* A, const void* const* B, void* const* C, uint8_t* ws,
                           cudaStream_t stream, double scale = 0.0) {
   const GemmPlan& g0 = s->gemms[members_in[0]];
   const KindInfo& k = kKinds[g0.kind];
+  const bool pair = !mixed && k.pair;
   const int out_bf16 = g0.desc.c_dtype == GOLDY_BF16 ? 1 : 0;
-  int ctas = 0;
-  goldy_status st = kernel_setup(d, g0.kind, out_bf16, 1, &ctas);
+  int ctas = 1;
+  const void* fn = nullptr;
+  goldy_status st = mixed ? set_kernel_setup(d, out_bf16) : kernel_setup(d, g0.kind, out_bf16, 1, &ctas);
   if (st != GOLDY_OK) return st;
-  static thread_local LaunchParams<kMaxFused> p;   // ~5 KB: keep it off the stack
+  fn = mixed ? kernel_fn_set(out_bf16) : kernel_fn(g0.kind, out_bf16, 1);
+  static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
   std::memset(&p, 0, sizeof(p));
   int64_t units = 0, cap = 0;
   // clusters need one split factor for every GEMM of the launch
   int split = g0.split;
+  int stage = 0;
   for (int j = 0; j < count; ++j) {
     const GemmPlan& gp = s->gemms[members_in[j]];
     units += gp.units;
     cap += std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(gp.variant).rc_div);
     if (gp.split != split) split = 0;
+    stage = std::max(stage, stage_bytes(kKinds[gp.kind]));
   }
   if (units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one launch");
   if (scale > 0.0) cap = std::max<int64_t>(1, int64_t(double(cap) * scale));
-  cap = std::min<int64_t>(cap, int64_t(ctas) * sms(d));
-  const int cluster = (!k.pair && split > 1 && cluster_feasible(d, g0.kind, out_bf16, 1, split)) ? split : 0;
-  const unsigned grid = k.pair ? pair_grid(units, cap) : launch_grid(units, cap, cluster);
-  // Units handed out by a counter (longest first) instead of round-robin:
-  // when the CTAs take several units each and the GEMMs' units differ in
-  // length (2x or more), a static order leaves the launch's end to the CTAs
-  // that drew the long ones (a launch of 868 six-K-block units and 15
-  // 93-K-block units: 123.6 -> 111.5 us for its set).  Equal units gain
-  // nothing and pay the counter (eight equal GEMMs: 17.9 -> 19.4 us).  Not
-  // with cluster-reduced split-K (a cluster's CTAs take the splits of one
-  // tile together) nor the pair kernel.
+  cap = whole ? int64_t(ctas) * sms(d) : std::min<int64_t>(cap, int64_t(ctas) * sms(d));
+  const int cluster =
+      (!mixed && !pair && split > 1 && cluster_feasible(d, g0.kind, out_bf16, 1, split)) ? split : 0;
+  const unsigned grid = pair ? pair_grid(units, cap) : launch_grid(units, cap, cluster);
+  // Units in equal shares, longest first, instead of round-robin in GEMM
+  // order: when the GEMMs' units differ in length, round-robin leaves the
+  // launch's end to the CTAs that drew the long ones.  (A counter in the
+  // workspace balanced as well, but its first read had to wait for the launch
+  // before, and the pair kernel had none.)  Not with cluster-reduced split-K:
+  // a cluster's CTAs take the splits of one tile together.
   int members[kMaxFused];
   for (int j = 0; j < count; ++j) members[j] = members_in[j];
-  auto unit_len = [&](int i) { return int64_t(s->gemms[i].k_blocks) / std::max(1, s->gemms[i].split); };
-  int64_t shortest = INT64_MAX, longest = 0;
-  for (int j = 0; j < count; ++j) {
-    shortest = std::min(shortest, unit_len(members[j]));
-    longest = std::max(longest, unit_len(members[j]));
+  if (cluster == 0) {
+    std::stable_sort(members, members + count,
+                     [&](int a, int b) { return unit_cost(s->gemms[a]) > unit_cost(s->gemms[b]); });
+    deal_units(p.shares, s, members, count, int(pair ? grid / 2 : grid));
   }
-  bool dyn = !k.pair && cluster == 0 && units > int64_t(grid) && ws != nullptr && longest >= 2 * shortest;
-  for (int j = 0; j < count && dyn; ++j) dyn = s->gemms[members[j]].ws_dyn_off != ~size_t(0);
-  if (dyn)
-    std::stable_sort(members, members + count, [&](int a, int b) { return unit_len(a) > unit_len(b); });
   units = 0;
   for (int j = 0; j < count; ++j) {
     const GemmPlan& gp = s->gemms[members[j]];
@@ -662,19 +729,15 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   p.err = d.err_word;
   p.wait_ns = t_wait_ns;
   p.early_loads = t_early;
+  p.late_trigger = t_late;
   p.stall_test = t_stall;
   t_stall = 0;
-  p.dyn = dyn ? reinterpret_cast<uint32_t*>(ws + s->gemms[members[0]].ws_dyn_off) : nullptr;
-  p.trace = trace_for(grid);
-  if (k.pair) {
-    cudaError_t e =
-        launch_kernel(kernel_fn(g0.kind, out_bf16, 1), grid, size_t(smem_bytes(k)), stream, &p, sizeof(p), 2);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernel (fused pair)");
-    return GOLDY_OK;
-  }
   p.cluster = cluster;
-  cudaError_t e =
-      launch_kernel(kernel_fn(g0.kind, out_bf16, 1), grid, size_t(smem_bytes(k)), stream, &p, sizeof(p), cluster);
+  p.stage_bytes = stage;
+  p.stages = mixed ? std::min(kSetMaxStages, kSetRing / stage) : 0;
+  p.trace = trace_for(grid);
+  cudaError_t e = launch_kernel(fn, grid, size_t(mixed ? kSetSmemBytes : smem_bytes(k)), stream, &p, sizeof(p),
+                                pair ? 2 : cluster);
   if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernel (fused)");
   return GOLDY_OK;
 }
@@ -728,6 +791,7 @@ struct RunOptionsReset {
     t_trace_used = 0;
     t_pdl = true;
     t_early = 0;
+    t_late = 0;
     t_wait_ns = 0;
     t_stall = 0;
   }
@@ -804,6 +868,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // first of them.
   struct LaunchSet {
     int group, slot, n, degenerate, wave;
+    bool mixed, whole;   // several kinds in one launch; grid cap the whole GPU
     double scale;     // grid-cap scale for heterogeneous fused waves (0: none)
     int rank;         // rank by FLOPs among the launches of its wave (0: largest)
     int prio;         // launch priority (kNoPriority: the stream's)
@@ -846,6 +911,59 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       }
     }
   }
+  // Fused plans of the dynamic logic: the launches of all waves and groups
+  // join into one launch of the pair kernel and one of the kernel over
+  // different single-CTA tile shapes (per output dtype, at most kMaxFused
+  // GEMMs each).  A wave's launches per kind paid a start each, and on one
+  // stream the stores of each waited for the launch before; in one persistent
+  // launch the units of every wave, dealt out longest first, keep the order of
+  // the plan's intent (large GEMMs first, small ones in the gaps).  A run that
+  // already is one launch stays as it is: its kind's own kernel is the better
+  // one there (deeper ring, split-K in a cluster).  Explicit schedules and the
+  // forced policies keep one launch per wave and kind.
+  if (fused && s->auto_plan && sets.size() > 1) {
+    std::vector<LaunchSet> joined;
+    joined.reserve(sets.size());
+    int singles[2] = {0, 0};               // launches of single-CTA kinds per output dtype
+    for (const LaunchSet& ls : sets)
+      if (!ls.degenerate && !kKinds[s->gemms[ls.members[0]].kind].pair)
+        ++singles[s->gemms[ls.members[0]].desc.c_dtype == GOLDY_BF16 ? 1 : 0];
+    for (const LaunchSet& ls : sets) {
+      const GemmPlan& g0 = s->gemms[ls.members[0]];
+      const bool pair = kKinds[g0.kind].pair != 0;
+      if (ls.degenerate) {
+        joined.push_back(ls);
+        joined.back().group = joined.back().wave = 0;
+        continue;
+      }
+      const bool mixed = !pair && singles[g0.desc.c_dtype == GOLDY_BF16 ? 1 : 0] > 1;
+      for (int j = 0; j < ls.n; ++j) {
+        const int i = ls.members[j];
+        size_t target = joined.size();
+        for (size_t t = 0; t < joined.size(); ++t) {
+          const GemmPlan& h0 = s->gemms[joined[t].members[0]];
+          if (!joined[t].degenerate && joined[t].n < kMaxFused && (kKinds[h0.kind].pair != 0) == pair &&
+              h0.desc.c_dtype == g0.desc.c_dtype) {
+            target = t;
+            break;
+          }
+        }
+        if (target == joined.size()) {
+          LaunchSet nw{};
+          nw.slot = ls.slot;
+          nw.prio = kNoPriority;
+          nw.mixed = mixed;
+          joined.push_back(nw);
+        }
+        LaunchSet& to = joined[target];
+        if (to.n > 0 && j == 0) to.whole = true;   // the members of several launches
+        to.members[to.n++] = i;
+        const goldy_gemm_desc& gd = s->gemms[i].desc;
+        to.flops += 2.0 * double(gd.M) * double(gd.N) * double(gd.K) * double(std::max<int64_t>(1, gd.batch));
+      }
+    }
+    sets.swap(joined);
+  }
   // Priority levels from the device's greatest (level 0) to its least.
   const int prio_step = d->prio_greatest <= d->prio_least ? 1 : -1;
   const int prio_levels = std::abs(d->prio_least - d->prio_greatest) + 1;
@@ -857,7 +975,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // the wave's launches are ranked by FLOPs into launch priorities, so the
   // largest gets the SMs first and smaller ones fill the SMs it frees in its
   // tail.
-  const bool soft_groups = fused && s->groups.size() > 1;
+  const bool soft_groups = fused && !s->auto_plan && s->groups.size() > 1;
   if (fused) {
     for (size_t t0 = 0; t0 < sets.size();) {
       size_t t1 = t0;
@@ -997,7 +1115,17 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // complete, so those runs keep the streams.
   int n_launches = 0;
   for (const LaunchSet& ls : sets) n_launches += ls.degenerate ? 0 : 1;
-  const bool one_stream = fused && t_early && n_launches >= 2;
+  const bool one_stream = fused && (t_early || s->auto_plan) && n_launches >= 2;
+  // A run of the dynamic logic without inputs_ready also goes out on
+  // streams[0] alone: its first launch waits for the work queued before the
+  // run, and lets the next launch start only after that (late_trigger), so the
+  // run's other launches may load their operands at once — every grid before
+  // the run has completed by then, and no launch of the run writes another's A
+  // or B.  Their epilogues still wait for the launch before.  (Not in a traced
+  // run, whose stamps are then those of one launch at a time, nor under a
+  // caller's own wait limit, which would come to cover the launch before.)
+  const bool chain = one_stream && !t_early && s->auto_plan && t_pdl && !t_trace && t_wait_ns == 0;
+  bool chained = false;
   if (one_stream) lead = sets.size();
   std::vector<size_t> order;
   order.reserve(sets.size());
@@ -1042,11 +1170,18 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       last_group[ls.slot] = ls.group;
       t_prio = ls.prio;
       t_started = order[t] == lead ? rt->started : nullptr;
-      if (ls.n == 1) {
+      if (chain && !ls.degenerate) {
+        t_late = chained ? 0 : 1;
+        t_early = chained ? 1 : 0;
+        chained = true;
+      }
+      // launches that follow one another on one stream each take the whole GPU
+      const bool whole = s->auto_plan && one_stream;
+      if (ls.n == 1 && !ls.mixed) {
         const int i = ls.members[0];
-        st = launch_gemm(*d, s->gemms[i], A[i], B[i], C[i], ws, stream, ls.scale);
+        st = launch_gemm(*d, s->gemms[i], A[i], B[i], C[i], ws, stream, whole ? 1e6 : ls.scale);
       } else {
-        st = launch_fused(*d, s, ls.members, ls.n, A, B, C, ws, stream, ls.scale);
+        st = launch_fused(*d, s, ls.members, ls.n, ls.mixed, ls.whole || whole, A, B, C, ws, stream, ls.scale);
       }
       t_prio = kNoPriority;
       t_started = nullptr;
