@@ -108,8 +108,19 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
   ptx::tc_fence_after();
   ptx::cluster_sync_all();                  // the peer's barriers and tensor memory are ready
   ptx::tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = ptx::uniform(*tmem_slot);
   const uint64_t wlim = p.wait_ns ? p.wait_ns : ptx::kWaitLimitNs;
+  // a wait of a whole role (warp); whichever lane gives up first raises the error
+  auto role_wait = [&](uint64_t* bar, uint32_t parity, int code) {
+    const bool done = ptx::mbar_wait(ptx::smem_u32(bar), parity, abort_flag, wlim);
+    if (!done) raise_error(p.err, abort_flag, code);
+    return ptx::warp_all(done);
+  };
+  auto role_wait_cluster = [&](uint64_t* bar, uint32_t parity, int code) {
+    const bool done = ptx::mbar_wait_cluster(ptx::smem_u32(bar), parity, abort_flag, wlim);
+    if (!done) raise_error(p.err, abort_flag, code);
+    return ptx::warp_all(done);
+  };
   UnitWalk walk(utab, n_gemms, p.shares.on, p.total_units, pair, n_pairs);
   // global memory only after the previous grid is done; in early mode the
   // load and MMA roles go ahead (see go_gemm_kernel) and the epilogue waits
@@ -121,36 +132,43 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
   if (p.late_trigger) ptx::griddep_launch_dependents();
   if (threadIdx.x == 64 && !epi_defer) trace_stamp(trace, kTrSetup);   // the first epilogue thread waits
 
+  // load and MMA roles as whole warps, one elected thread issuing: see
+  // go_gemm_kernel
   if (warp == 0) {
-    if (lane == 0) {
+    {
       // ------------------------------------------------------------ producer
+      const bool leader = ptx::elect_one();
       int stage = 0;
       uint32_t phase = 0, issued = 0, last_phase = 0;
       bool ok = true;
-      while (ok && walk.next()) {
-        const UnitCoord c = walk.coord();
+      while (ok && ptx::warp_all(walk.next())) {
+        const UnitCoord c = walk.coord().uniform();
         const void* ta = &p.tmap_a[c.g];
         const void* tb = &p.tmap_b[c.g];
         const int m0 = c.tm * 256 + int(rank) * 128;
-        const bool narrow = utab[c.g].n - c.tn * 256 <= 128;
+        const bool narrow = ptx::uniform(utab[c.g].n) - c.tn * 256 <= 128;
         const int n0 = c.tn * 256 + int(rank) * (narrow ? HALF_N / 2 : HALF_N);
         const uint32_t pair_bytes = narrow ? 2 * (A_BYTES + B_BYTES / 2) : 2 * STAGE_BYTES;
         for (int kb = c.kb0; kb < c.kb1; ++kb) {
           // only a slot filled before is waited for (see go_gemm_kernel)
-          if ((issued >> stage & 1) && !ptx::mbar_wait(ptx::smem_u32(&empty[stage]), phase ^ 1, abort_flag, wlim)) {
+          if ((issued >> stage & 1) &&
+              !role_wait(&empty[stage], phase ^ 1, kErrProducerWait)) {
             ok = false;
             break;
           }
           const uint32_t fb_local = ptx::smem_u32(&full[stage]);
           const uint32_t fb = ptx::map_to_rank(fb_local, 0);      // the even CTA's barrier
-          if (lead) ptx::mbar_arrive_expect_tx(fb_local, pair_bytes);
           const uint32_t xs = tiles_base + stage * STAGE_BYTES;
           const uint32_t ys = xs + A_BYTES;
           const int k0 = kb * 64;
-          ptx::tma_load_3d_pair(xs, ta, fb, k0, m0, c.b);
-          ptx::tma_load_3d_pair(ys, tb, fb, n0, k0, c.b);
-          if (!narrow) ptx::tma_load_3d_pair(ys + 8192, tb, fb, n0 + 64, k0, c.b);
-          if (issued == 0) trace_stamp(trace, kTrFirstLoad);
+          if (leader) {
+            if (lead) ptx::mbar_arrive_expect_tx(fb_local, pair_bytes);
+            ptx::tma_load_3d_pair(xs, ta, fb, k0, m0, c.b);
+            ptx::tma_load_3d_pair(ys, tb, fb, n0, k0, c.b);
+            if (!narrow) ptx::tma_load_3d_pair(ys + 8192, tb, fb, n0 + 64, k0, c.b);
+          }
+          __syncwarp();
+          if (issued == 0 && lane == 0) trace_stamp(trace, kTrFirstLoad);
           issued |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == STAGES) {
@@ -159,13 +177,12 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
           }
         }
       }
-      if (!ok) raise_error(p.err, abort_flag, kErrProducerWait);
       // every slot this CTA filled must have been released by the pair MMA
       // (so the even CTA's commits to this CTA's barriers have landed, and
       // the peer's loads into the even CTA's slots are done) before leaving
       const uint64_t t0 = ptx::global_timer();
       for (int s = 0; s < STAGES; ++s) {
-        if (!(issued >> s & 1)) continue;
+        if (!leader || !(issued >> s & 1)) continue;
         const uint32_t bar = ptx::smem_u32(&empty[s]);
         const uint32_t par = (last_phase >> s) & 1;
         while (!ptx::mbar_try_wait(bar, par)) {
@@ -177,58 +194,62 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && lead) {
+    if (lead) {
       // ------------------------------------------------- MMA issuer (even CTA)
+      const bool leader = ptx::elect_one();
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, acc_used = 0;
       bool ok = true, any = false, first = true;
-      while (ok && walk.next()) {
-        const UnitCoord c = walk.coord();
+      while (ok && ptx::warp_all(walk.next())) {
+        const UnitCoord c = walk.coord().uniform();
         // both CTAs drained this accumulator (the odd CTA signals with a
         // cluster-scope release, so wait with a cluster-scope acquire); the
         // first use of an accumulator needs no wait
         if ((acc_used >> acc & 1) &&
-            !ptx::mbar_wait_cluster(ptx::smem_u32(&tempty[acc]), acc_phase ^ 1, abort_flag, wlim)) {
+            !role_wait_cluster(&tempty[acc], acc_phase ^ 1, kErrMmaWait)) {
           ok = false;
           break;
         }
         acc_used |= 1u << acc;
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + uint32_t(acc * 256);
-        const uint32_t idesc = utab[c.g].n - c.tn * 256 <= 128 ? IDESC_NARROW : IDESC;
+        const uint32_t idesc = ptx::uniform(utab[c.g].n) - c.tn * 256 <= 128 ? IDESC_NARROW : IDESC;
         for (int kb = c.kb0; kb < c.kb1; ++kb) {
-          if (!ptx::mbar_wait(ptx::smem_u32(&full[stage]), phase, abort_flag, wlim)) {
+          if (!role_wait(&full[stage], phase, kErrMmaWait)) {
             ok = false;
             break;
           }
           ptx::tc_fence_after();
-          if (!any) trace_stamp(trace, kTrFirstFull);
+          if (!any && lane == 0) trace_stamp(trace, kTrFirstFull);
           const uint32_t xs = tiles_base + stage * STAGE_BYTES;
           const uint32_t ys = xs + A_BYTES;
+          if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t adesc = ptx::make_sdesc_sw128(xs + kk * KMAJ_STEP, 16, 1024);
-            const uint64_t bdesc = ptx::make_sdesc_sw128(ys + kk * MNMAJ_STEP, MNMAJ_LBO, 1024);
-            ptx::mma_bf16_pair(d_tmem, adesc, bdesc, idesc, (kb > c.kb0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < 4; ++kk) {
+              const uint64_t adesc = ptx::make_sdesc_sw128(xs + kk * KMAJ_STEP, 16, 1024);
+              const uint64_t bdesc = ptx::make_sdesc_sw128(ys + kk * MNMAJ_STEP, MNMAJ_LBO, 1024);
+              ptx::mma_bf16_pair(d_tmem, adesc, bdesc, idesc, (kb > c.kb0 || kk > 0) ? 1u : 0u);
+            }
+            ptx::mma_commit_pair_multicast(ptx::smem_u32(&empty[stage]), 0x3);
           }
+          __syncwarp();
           any = true;
-          ptx::mma_commit_pair_multicast(ptx::smem_u32(&empty[stage]), 0x3);
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1;
           }
         }
         if (!ok) break;
-        ptx::mma_commit_pair_multicast(ptx::smem_u32(&tfull[acc]), 0x3);
-        if (first) trace_stamp(trace, kTrFirstMmaDone);
+        if (leader) ptx::mma_commit_pair_multicast(ptx::smem_u32(&tfull[acc]), 0x3);
+        __syncwarp();
+        if (first && lane == 0) trace_stamp(trace, kTrFirstMmaDone);
         first = false;
         if (++acc == ACC) {
           acc = 0;
           acc_phase ^= 1;
         }
       }
-      if (!ok) {
-        raise_error(p.err, abort_flag, kErrMmaWait);
+      if (!ok && leader) {
         if (any) {
           ptx::mma_commit_pair_multicast(ptx::smem_u32(drain), 0x1);
           ptx::mbar_wait(ptx::smem_u32(drain), 0, nullptr);
@@ -256,7 +277,9 @@ __global__ void __launch_bounds__(192, 1) go_gemm_pair_kernel(const __grid_const
       const UnitCoord c = walk.coord();
       const GemmWork w = p.g[c.g];                 // read while the accumulator is computed
       const CView cv = c_view<OUT_BF16>(w, c.b);
-      bool ok = ptx::mbar_wait(ptx::smem_u32(&tfull[acc]), acc_phase, abort_flag, wlim);
+      // (a little longer than the other roles wait: what they wait for is what
+      // this wait hangs on, so the role that is stuck reports)
+      bool ok = ptx::mbar_wait(ptx::smem_u32(&tfull[acc]), acc_phase, abort_flag, wlim + wlim / 8);
       ok = ptx::named_bar_and(1, 128, ok);
       if (!ok) {
         if (et == 0) raise_error(p.err, abort_flag, kErrEpilogueWait);

@@ -97,8 +97,14 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = ptx::uniform(*tmem_slot);
   const uint64_t wlim = p.wait_ns ? p.wait_ns : ptx::kWaitLimitNs;
+  // a wait of a whole role (warp); whichever lane gives up first raises the error
+  auto role_wait = [&](uint64_t* bar, uint32_t parity, int code) {
+    const bool done = ptx::mbar_wait(ptx::smem_u32(bar), parity, abort_flag, wlim);
+    if (!done) raise_error(p.err, abort_flag, code);
+    return ptx::warp_all(done);
+  };
   UnitWalk walk(utab, n_gemms, p.shares.on, p.total_units, int(blockIdx.x), int(gridDim.x));
   if (threadIdx.x == 0) trace_stamp(trace, kTrPreWait);
   // where each role waits for the previous grid: see go_gemm_kernel
@@ -108,19 +114,22 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
   if (p.late_trigger) ptx::griddep_launch_dependents();
   if (threadIdx.x == 64 && !epi_defer) trace_stamp(trace, kTrSetup);
 
+  // load and MMA roles as whole warps, one elected thread issuing: see
+  // go_gemm_kernel
   if (warp == 0) {
-    if (lane == 0) {
+    {
       // ------------------------------------------------------------ producer
+      const bool leader = ptx::elect_one();
       int stage = 0;
       uint32_t phase = 0, issued = 0, last_phase = 0;
       bool ok = true, stalled = false;
-      while (ok && !stalled && walk.next()) {
-        if (issued == 0) trace_stamp(trace, kTrProducerGo);
-        const UnitCoord c = walk.coord();
+      while (ok && !stalled && ptx::warp_all(walk.next())) {
+        if (issued == 0 && lane == 0) trace_stamp(trace, kTrProducerGo);
+        const UnitCoord c = walk.coord().uniform();
         const void* ta = &p.tmap_a[c.g];
         const void* tb = &p.tmap_b[c.g];
-        const int mma_n = utab[c.g].mma_n;
-        const bool swap = utab[c.g].swap != 0;
+        const int mma_n = ptx::uniform(utab[c.g].mma_n);
+        const bool swap = ptx::uniform(utab[c.g].swap) != 0;
         const uint32_t bytes = X_BYTES + uint32_t(mma_n) * 128u;
         const int m0 = c.tm * (swap ? mma_n : 128);
         const int n0 = c.tn * (swap ? 128 : mma_n);
@@ -129,7 +138,8 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
         const uint32_t a_off = swap ? X_BYTES : 0u, b_off = swap ? 0u : X_BYTES;
         for (int kb = c.kb0; kb < c.kb1; ++kb) {
           // only a slot filled before is waited for (see go_gemm_kernel)
-          if ((issued >> stage & 1) && !ptx::mbar_wait(ptx::smem_u32(&empty[stage]), phase ^ 1, abort_flag, wlim)) {
+          if ((issued >> stage & 1) &&
+              !role_wait(&empty[stage], phase ^ 1, kErrProducerWait)) {
             ok = false;
             break;
           }
@@ -142,13 +152,16 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
             break;
           }
           const uint32_t fb = ptx::smem_u32(&full[stage]);
-          ptx::mbar_arrive_expect_tx(fb, bytes);
           const uint32_t base = tiles_base + uint32_t(stage) * stage_bytes;
           const int k0 = kb * 64;
-          ptx::tma_load_3d(base + a_off, ta, fb, k0, m0, c.b);
-          for (int j = 0; j < boxes; ++j)
-            ptx::tma_load_3d(base + b_off + uint32_t(j) * 8192u, tb, fb, n0 + 64 * j, k0, c.b);
-          if (issued == 0) trace_stamp(trace, kTrFirstLoad);
+          if (leader) {
+            ptx::mbar_arrive_expect_tx(fb, bytes);
+            ptx::tma_load_3d(base + a_off, ta, fb, k0, m0, c.b);
+            for (int j = 0; j < boxes; ++j)
+              ptx::tma_load_3d(base + b_off + uint32_t(j) * 8192u, tb, fb, n0 + 64 * j, k0, c.b);
+          }
+          __syncwarp();
+          if (issued == 0 && lane == 0) trace_stamp(trace, kTrFirstLoad);
           issued |= 1u << stage;
           last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
           if (++stage == stages) {
@@ -157,30 +170,30 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
           }
         }
       }
-      if (!ok) {
-        raise_error(p.err, abort_flag, kErrProducerWait);
+      if (!ok && leader) {
         // let every copy this thread started land before the CTA can exit
         for (int s = 0; s < stages; ++s)
           if (issued >> s & 1) ptx::mbar_wait(ptx::smem_u32(&full[s]), (last_phase >> s) & 1, nullptr);
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       // ---------------------------------------------------------- MMA issuer
+      const bool leader = ptx::elect_one();
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, acc_used = 0;
       bool ok = true, any = false, first = true;
-      while (ok && walk.next()) {
-        const UnitCoord c = walk.coord();
-        const int mma_n = utab[c.g].mma_n;
-        const bool swap = utab[c.g].swap != 0;
+      while (ok && ptx::warp_all(walk.next())) {
+        const UnitCoord c = walk.coord().uniform();
+        const int mma_n = ptx::uniform(utab[c.g].mma_n);
+        const bool swap = ptx::uniform(utab[c.g].swap) != 0;
         // untransposed: MMA-A = A tile (K-major), MMA-B = B tile (N-major);
         // transposed: MMA-A = B tile (N-major), MMA-B = A tile (K-major)
         const uint32_t idesc = ptx::make_idesc_bf16(128, mma_n, swap ? 1 : 0, swap ? 0 : 1);
         const uint32_t a_step = swap ? MNMAJ_STEP : KMAJ_STEP, b_step = swap ? KMAJ_STEP : MNMAJ_STEP;
         const uint32_t a_lbo = swap ? MNMAJ_LBO : 16u, b_lbo = swap ? 16u : MNMAJ_LBO;
         if ((acc_used >> acc & 1) &&
-            !ptx::mbar_wait(ptx::smem_u32(&tempty[acc]), acc_phase ^ 1, abort_flag, wlim)) {
+            !role_wait(&tempty[acc], acc_phase ^ 1, kErrMmaWait)) {
           ok = false;
           break;
         }
@@ -188,38 +201,41 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + uint32_t(acc * ACC_COLS);
         for (int kb = c.kb0; kb < c.kb1; ++kb) {
-          if (!ptx::mbar_wait(ptx::smem_u32(&full[stage]), phase, abort_flag, wlim)) {
+          if (!role_wait(&full[stage], phase, kErrMmaWait)) {
             ok = false;
             break;
           }
           ptx::tc_fence_after();
-          if (!any) trace_stamp(trace, kTrFirstFull);
+          if (!any && lane == 0) trace_stamp(trace, kTrFirstFull);
           const uint32_t xs = tiles_base + uint32_t(stage) * stage_bytes;
           const uint32_t ys = xs + X_BYTES;
+          if (leader) {
 #pragma unroll
-          for (uint32_t kk = 0; kk < 4; ++kk) {
-            const uint64_t adesc = ptx::make_sdesc_sw128(xs + kk * a_step, a_lbo, 1024);
-            const uint64_t bdesc = ptx::make_sdesc_sw128(ys + kk * b_step, b_lbo, 1024);
-            ptx::mma_bf16(d_tmem, adesc, bdesc, idesc, (kb > c.kb0 || kk > 0) ? 1u : 0u);
+            for (uint32_t kk = 0; kk < 4; ++kk) {
+              const uint64_t adesc = ptx::make_sdesc_sw128(xs + kk * a_step, a_lbo, 1024);
+              const uint64_t bdesc = ptx::make_sdesc_sw128(ys + kk * b_step, b_lbo, 1024);
+              ptx::mma_bf16(d_tmem, adesc, bdesc, idesc, (kb > c.kb0 || kk > 0) ? 1u : 0u);
+            }
+            ptx::mma_commit(ptx::smem_u32(&empty[stage]));   // frees the slot when these MMAs finish
           }
+          __syncwarp();
           any = true;
-          ptx::mma_commit(ptx::smem_u32(&empty[stage]));   // frees the slot when these MMAs finish
           if (++stage == stages) {
             stage = 0;
             phase ^= 1;
           }
         }
         if (!ok) break;
-        ptx::mma_commit(ptx::smem_u32(&tfull[acc]));        // accumulator complete
-        if (first) trace_stamp(trace, kTrFirstMmaDone);
+        if (leader) ptx::mma_commit(ptx::smem_u32(&tfull[acc]));   // accumulator complete
+        __syncwarp();
+        if (first && lane == 0) trace_stamp(trace, kTrFirstMmaDone);
         first = false;
         if (++acc == ACC) {
           acc = 0;
           acc_phase ^= 1;
         }
       }
-      if (!ok) {
-        raise_error(p.err, abort_flag, kErrMmaWait);
+      if (!ok && leader) {
         if (any) {
           ptx::mma_commit(ptx::smem_u32(drain));
           ptx::mbar_wait(ptx::smem_u32(drain), 0, nullptr);
@@ -247,7 +263,9 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
       const UnitCoord c = walk.coord();
       const GemmWork w = p.g[c.g];          // read while the accumulator is computed
       const CView cv = c_view<OUT_BF16>(w, c.b);
-      bool ok = ptx::mbar_wait(ptx::smem_u32(&tfull[acc]), acc_phase, abort_flag, wlim);
+      // (a little longer than the other roles wait: what they wait for is what
+      // this wait hangs on, so the role that is stuck reports)
+      bool ok = ptx::mbar_wait(ptx::smem_u32(&tfull[acc]), acc_phase, abort_flag, wlim + wlim / 8);
       ok = ptx::named_bar_and(1, 128, ok);
       if (!ok) {
         if (et == 0) raise_error(p.err, abort_flag, kErrEpilogueWait);

@@ -26,6 +26,20 @@ __device__ __forceinline__ uint64_t global_timer() {
   return t;
 }
 
+// One thread of a converged warp (the same one each time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+  return pred != 0;
+}
+// Lane 0's value, so that the compiler knows it is the same in every lane.
+template <typename T>
+__device__ __forceinline__ T uniform(T v) {
+  return __shfl_sync(0xffffffffu, v, 0);
+}
+// Does every lane say so?
+__device__ __forceinline__ bool warp_all(bool v) { return __all_sync(0xffffffffu, v) != 0; }
+
 // ---- mbarrier --------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
