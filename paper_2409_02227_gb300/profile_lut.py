@@ -46,7 +46,7 @@ With ``--dataset FILE`` it instead records the CD predictor's training set
 with the table's GO-Kernel for that CD.
 
 Usage (on a GPU):  python -m paper_2409_02227_gb300.profile_lut --out DIR
-                   [--configs] [--sweep] [--keys lm,ln,lk,out ...]
+                   [--configs] [--sweep] [--range] [--keys lm,ln,lk,out ...]
                    python -m paper_2409_02227_gb300.profile_lut --dataset FILE
 """
 from __future__ import annotations
@@ -453,6 +453,21 @@ def sweep_keys() -> List[Tuple[int, int, int, int]]:
     return sorted(keys)
 
 
+def range_keys() -> List[Tuple[int, int, int, int]]:
+    """Every bucket of the declared ranges — M in [16, 4096], N and K in [256,
+    8192], fp32 and bf16 out — and of attention B-GEMMs (sequences of 128 to
+    2048, 16 or 32 heads of dimension 128) in both dtypes.  A table without a
+    bucket falls back to the nearest stored one of the same dtype, which can
+    lie far away: with the bf16 buckets of two workloads only, two GEMMs of
+    4096 x 8192 x 8192 ran on 64-row transposed tiles (2720 us; 683 us with
+    their own bucket)."""
+    keys = set()
+    for out in (G.GOLDY_BF16, G.GOLDY_F32):
+        keys |= {(m, n, k, out) for m in range(4, 13) for n in range(8, 14) for k in range(8, 14)}
+        keys |= {key for l in range(7, 12) for h in (4, 5) for key in ((l + h, l, 7, out), (l + h, 7, l, out))}
+    return sorted(keys)
+
+
 def bucket_of(M: int, N: int, K: int, out: int) -> Tuple[int, int, int, int]:
     key = G.goldy_bucket_key(G.desc(M, N, K, out, lda=max(8, -(-K // 8) * 8), ldb=max(8, -(-N // 8) * 8)))
     return (key >> 24) & 0xFF, (key >> 16) & 0xFF, (key >> 8) & 0xFF, key & 0xFF
@@ -478,6 +493,8 @@ def main(argv=None) -> int:
                          "a co-run log, under the current preferred-CD and co-run rules")
     ap.add_argument("--configs", action="store_true", help="buckets of the fixed workload sets")
     ap.add_argument("--sweep", action="store_true", help="buckets of the 64 randomized sets")
+    ap.add_argument("--range", action="store_true",
+                    help="every bucket of the declared ranges (M 16-4096, N and K 256-8192, attention), both dtypes")
     ap.add_argument("--keys", nargs="*", default=[], help="extra buckets lm,ln,lk,out")
     ap.add_argument("--time-budget", type=float, default=1e9, help="stop starting buckets after this many seconds")
     ap.add_argument("--launch", choices=["fused", "streams"], default="fused",
@@ -507,6 +524,8 @@ def main(argv=None) -> int:
         keys += config_keys()
     if args.sweep:
         keys += sweep_keys()
+    if args.range:
+        keys += range_keys()
     if args.scaling_keys:
         keys += sorted({bucket_of(*sh) for sh in wl.scaling_study_shapes()})
     if args.batched_keys:
