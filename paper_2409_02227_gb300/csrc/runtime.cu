@@ -571,15 +571,42 @@ unsigned long long* trace_for(unsigned grid) {
   return region;
 }
 
+// The kind that runs a launch planned for `kind`.  With inputs_ready the next
+// run's CTAs may load and multiply while this run's wait for their stores, if
+// an SM has room for them: a launch of at most two CTAs' worth of units per SM
+// therefore takes the two-per-SM kind of the same tile shape (same K split,
+// same order of sums: the same bytes), so that a run no longer starts when the
+// one before leaves its SMs.  Measured back to back: four layers of eight 32 x
+// 4096 x 1024 59.1 -> 45.7 us, of four 128 x 1024 x 4096 split 4 41.6 -> 36.1
+// us, 753 x 1152 x 704 and a smaller one 6.6 -> 4.4 us.  A launch whose splits
+// reduce in clusters only when two runs do not fit side by side anyway: the
+// two-per-SM kinds have no room for pushed partials (two 256 x 256 x 512 split
+// 4, 64 CTAs: 3.06 -> 3.90 us).  256-wide tiles keep their deeper ring.
+int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, int split) {
+  if (!t_early || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 || kKinds[kind].mma_n > 128) return kind;
+  const int twin = kind + 1;
+  static_assert(kKinds[1].mma_n == kKinds[0].mma_n && kKinds[3].mma_n == kKinds[2].mma_n &&
+                    kKinds[7].mma_n == kKinds[6].mma_n && kKinds[9].mma_n == kKinds[8].mma_n &&
+                    kKinds[1].ctas_per_sm == 2 && kKinds[3].ctas_per_sm == 2 && kKinds[7].ctas_per_sm == 2 &&
+                    kKinds[9].ctas_per_sm == 2,
+                "a full kind is followed by the half kind of its tile shape");
+  if (units > 2 * int64_t(sms(d))) return kind;
+  int ctas = 0;   // (the set-up also readies the kernel for the cluster query)
+  if (kernel_setup(d, twin, out_bf16, fused, &ctas) != GOLDY_OK || ctas < 2) return kind;
+  if (split > 1 && (2 * units <= sms(d) || !cluster_feasible(d, twin, out_bf16, fused, split))) return kind;
+  return twin;
+}
+
 // scale > 0: the launch's grid cap is its variant's cap times `scale` (set for
 // heterogeneous fused waves, see goldy_run_ex), at most the whole GPU.
 goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, const void* B, void* C, uint8_t* ws,
                          cudaStream_t stream, double scale = 0.0) {
   if (degenerate(gp)) return launch_degenerate(gp, C, stream);
-  const KindInfo& k = kKinds[gp.kind];
   const int out_bf16 = gp.desc.c_dtype == GOLDY_BF16 ? 1 : 0;
+  const int kind = run_kind(d, gp.kind, out_bf16, 0, gp.units, gp.split);
+  const KindInfo& k = kKinds[kind];
   int ctas = 0;
-  goldy_status st = kernel_setup(d, gp.kind, out_bf16, 0, &ctas);
+  goldy_status st = kernel_setup(d, kind, out_bf16, 0, &ctas);
   if (st != GOLDY_OK) return st;
   if (gp.units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one GEMM");
 
@@ -603,16 +630,16 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
     const unsigned grid = pair_grid(gp.units, cap);
     p.trace = trace_for(grid);
     cudaError_t e =
-        launch_kernel(kernel_fn(gp.kind, out_bf16, 0), grid, size_t(smem_bytes(k)), stream, &p, sizeof(p), 2);
+        launch_kernel(kernel_fn(kind, out_bf16, 0), grid, size_t(smem_bytes(k)), stream, &p, sizeof(p), 2);
     if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernel (pair)");
     return GOLDY_OK;
   }
-  const int cluster = (gp.split > 1 && cluster_feasible(d, gp.kind, out_bf16, 0, gp.split)) ? gp.split : 0;
+  const int cluster = (gp.split > 1 && cluster_feasible(d, kind, out_bf16, 0, gp.split)) ? gp.split : 0;
   p.cluster = cluster;
   const unsigned grid = launch_grid(gp.units, cap, cluster);
   p.trace = trace_for(grid);
   cudaError_t e =
-      launch_kernel(kernel_fn(gp.kind, out_bf16, 0), grid, size_t(smem_bytes(k)), stream, &p, sizeof(p), cluster);
+      launch_kernel(kernel_fn(kind, out_bf16, 0), grid, size_t(smem_bytes(k)), stream, &p, sizeof(p), cluster);
   if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernel");
   return GOLDY_OK;
 }
@@ -677,32 +704,36 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
                           bool whole, const void* const* A, const void* const* B, void* const* C, uint8_t* ws,
                           cudaStream_t stream, double scale = 0.0) {
   const GemmPlan& g0 = s->gemms[members_in[0]];
-  const KindInfo& k = kKinds[g0.kind];
-  const bool pair = !mixed && k.pair;
   const int out_bf16 = g0.desc.c_dtype == GOLDY_BF16 ? 1 : 0;
-  int ctas = 1;
-  const void* fn = nullptr;
-  goldy_status st = mixed ? set_kernel_setup(d, out_bf16) : kernel_setup(d, g0.kind, out_bf16, 1, &ctas);
-  if (st != GOLDY_OK) return st;
-  fn = mixed ? kernel_fn_set(out_bf16) : kernel_fn(g0.kind, out_bf16, 1);
-  static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
-  std::memset(&p, 0, sizeof(p));
-  int64_t units = 0, cap = 0;
+  int64_t units = 0;
   // clusters need one split factor for every GEMM of the launch
   int split = g0.split;
+  for (int j = 0; j < count; ++j) {
+    units += s->gemms[members_in[j]].units;
+    if (s->gemms[members_in[j]].split != split) split = 0;
+  }
+  const int kind = mixed ? g0.kind : run_kind(d, g0.kind, out_bf16, 1, units, split);
+  const KindInfo& k = kKinds[kind];
+  const bool pair = !mixed && k.pair;
+  int ctas = 1;
+  const void* fn = nullptr;
+  goldy_status st = mixed ? set_kernel_setup(d, out_bf16) : kernel_setup(d, kind, out_bf16, 1, &ctas);
+  if (st != GOLDY_OK) return st;
+  fn = mixed ? kernel_fn_set(out_bf16) : kernel_fn(kind, out_bf16, 1);
+  static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
+  std::memset(&p, 0, sizeof(p));
+  int64_t cap = 0;
   int stage = 0;
   for (int j = 0; j < count; ++j) {
     const GemmPlan& gp = s->gemms[members_in[j]];
-    units += gp.units;
     cap += std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(gp.variant).rc_div);
-    if (gp.split != split) split = 0;
     stage = std::max(stage, stage_bytes(kKinds[gp.kind]));
   }
   if (units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one launch");
   if (scale > 0.0) cap = std::max<int64_t>(1, int64_t(double(cap) * scale));
   cap = whole ? int64_t(ctas) * sms(d) : std::min<int64_t>(cap, int64_t(ctas) * sms(d));
   const int cluster =
-      (!mixed && !pair && split > 1 && cluster_feasible(d, g0.kind, out_bf16, 1, split)) ? split : 0;
+      (!mixed && !pair && split > 1 && cluster_feasible(d, kind, out_bf16, 1, split)) ? split : 0;
   const unsigned grid = pair ? pair_grid(units, cap) : launch_grid(units, cap, cluster);
   // Units in equal shares, longest first, instead of round-robin in GEMM
   // order: when the GEMMs' units differ in length, round-robin leaves the
