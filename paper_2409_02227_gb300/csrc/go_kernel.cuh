@@ -84,7 +84,7 @@ __device__ __forceinline__ CView c_view(const GemmWork& w, int b) {
 // takes part in, then units first[g][b] .. first[g][b + 1] - 1 behind those.
 // The host deals the units out, longest GEMMs first, so that every bin gets
 // the same work (assign_units); with one GEMM per launch the units are equal
-// and go round-robin.  (Whole rounds keep the bins on neighbouring tiles:
+// and go round-robin (`on` = 2: back and forth).  (Whole rounds keep the bins on neighbouring tiles:
 // with one contiguous range per bin the operand panels in use at a time are
 // three times as many, bench set 50.4 -> 51.4 us.)
 constexpr int kMaxBins = 160;
@@ -121,7 +121,7 @@ struct LaunchParams {
   int32_t late_trigger;       // 1: let the next launch on the stream start only once this one is past its wait
                               // for the grid before (early_loads is 0 then): the next launch, of the same run,
                               // may then load its A and B at once, since every grid before the run has completed
-  int32_t stage_bytes, stages;   // operand ring of a launch that mixes tile shapes
+  int32_t stage_bytes, stages, acc_stages;   // ring and accumulators of a launch that mixes tile shapes
   UnitShares<MAXG> shares;    // on: the units of each CTA (pair); off: round-robin
 };
 
@@ -194,7 +194,7 @@ __device__ __forceinline__ void fill_unit_table(UnitTable* t, const LaunchParams
     e.n = p.g[g].n;
     e.rounds = e.lo = e.hi = 0;
     if constexpr (MAXG > 1) {
-      if (p.shares.on) {
+      if (p.shares.on == 1) {
         e.rounds = int(p.shares.rounds[g]);
         e.lo = e.unit_begin + int(p.shares.first[g][bin]);
         e.hi = e.unit_begin + int(p.shares.first[g][bin + 1]);
@@ -214,13 +214,17 @@ struct UnitWalk {
   int g, u, rounds;     // rounds: whole rounds left of GEMM g; -1: in the units behind them
 
   __device__ __forceinline__ UnitWalk(const UnitTable* tab, int n, int shares_on, int total_units, int bin, int bins)
-      : t(tab), n_gemms(n), shares(shares_on), total(total_units), bin(bin), step(bins), g(shares_on ? -1 : 0),
-        u(bin - bins), rounds(-1) {}
+      : t(tab), n_gemms(n), shares(shares_on), total(total_units), bin(bin), step(bins), g(shares_on == 1 ? -1 : 0),
+        u(shares_on == 2 ? -1 - bin : bin - bins), rounds(-1) {}
 
   // Move to the next unit; false when there is none.
   __device__ __forceinline__ bool next() {
-    if (!shares) {
-      u += step;
+    if (shares != 1) {
+      // round-robin; back and forth: every other round in reverse
+      if (shares == 0)
+        u += step;
+      else
+        u += (rounds = ~rounds) ? 2 * (step - bin) - 1 : 2 * bin + 1;
       return u < total;
     }
     for (;;) {
@@ -246,7 +250,7 @@ struct UnitWalk {
   __device__ __forceinline__ UnitCoord coord() const {
     UnitCoord c;
     int gi = g;
-    if (!shares)
+    if (shares != 1)
 #pragma unroll 1
       while (gi + 1 < n_gemms && u >= t[gi + 1].unit_begin) ++gi;
     const UnitTable& w = t[gi];

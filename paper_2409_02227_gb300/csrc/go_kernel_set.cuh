@@ -14,33 +14,41 @@
 // and K split, so the bytes are those of the GEMM run alone.  Split-K partials
 // go through the workspace, the last split to arrive sums them in split order.
 //
-// One CTA per SM: tensor memory holds two accumulators of 256 columns whatever
-// the tile's width; the operand ring is cut into stages of the launch's widest
-// tile (192 KB: 4 stages of 48 KB up to 8 of 24 KB or less).
+// CTAS = 1, one CTA per SM: tensor memory holds two accumulators of 256 columns
+// whatever the tile's width; the operand ring is cut into stages of the
+// launch's widest tile (192 KB: 4 stages of 48 KB up to 8 of 24 KB or less).
+// CTAS = 2, two per SM, for runs with inputs_ready: half the ring and half the
+// tensor memory (two accumulators of 128 columns, or one of 256 when the launch
+// has tiles that wide), no staging buffers (tiles other than a CTA's last are
+// stored from registers), so that the next run's CTAs load and multiply while
+// this run's finish.  The units, sorted longest first, go to the CTAs back and
+// forth (0 .. n-1, n-1 .. 0, ...), which balances the few units a CTA gets.
 #pragma once
 
 #include "go_kernel.cuh"
 
 namespace goldy {
 
-constexpr int kSetRingBytes = 4 * 49152;
 constexpr int kSetStages = 8;              // barriers for the most stages a launch may use
+template <int CTAS>
+constexpr int kSetRingBytes = 4 * 49152 / CTAS;
 
-template <bool OUT_BF16, int MAXG>
-__global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_constant__ LaunchParams<MAXG> p) {
-  constexpr int ACC = 2;
-  constexpr int ACC_COLS = 256;
+template <bool OUT_BF16, int MAXG, int CTAS>
+__global__ void __launch_bounds__(192, CTAS) go_gemm_set_kernel(const __grid_constant__ LaunchParams<MAXG> p) {
+  constexpr int ACC = 2;                             // accumulators at most (p.acc_stages of them in use)
+  const int acc_stages = CTAS == 1 ? ACC : p.acc_stages;
+  const uint32_t acc_cols = CTAS == 1 ? 256u : 256u / uint32_t(p.acc_stages);
   constexpr uint32_t X_BYTES = 128 * 64 * 2;         // MMA operand A: 128 rows x 64 K
-  constexpr uint32_t TMEM_COLS = 512;
+  constexpr uint32_t TMEM_COLS = 512 / CTAS;
   constexpr uint32_t KMAJ_STEP = 32;                 // bytes per 16 K elements, K-major
   constexpr uint32_t MNMAJ_STEP = 2048;              // bytes per 16 K rows, N-major
   constexpr uint32_t MNMAJ_LBO = 64 * 128;           // bytes between 64-wide N chunks
-  constexpr int STAGING_BYTES = 2 * 16384;
-  static_assert(kSetRingBytes >= 128 * ACC_COLS * 4, "the ring holds a whole tile");
+  constexpr int STAGING_BYTES = CTAS == 1 ? 2 * 16384 : 0;
+  constexpr int RING_BYTES = kSetRingBytes<CTAS>;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kSetRingBytes + STAGING_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES + STAGING_BYTES);
   uint64_t* full = bars;
   uint64_t* empty = bars + kSetStages;
   uint64_t* tfull = bars + 2 * kSetStages;
@@ -199,7 +207,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
         }
         acc_used |= 1u << acc;
         ptx::tc_fence_after();
-        const uint32_t d_tmem = tmem_base + uint32_t(acc * ACC_COLS);
+        const uint32_t d_tmem = tmem_base + uint32_t(acc) * acc_cols;
         for (int kb = c.kb0; kb < c.kb1; ++kb) {
           if (!role_wait(&full[stage], phase, kErrMmaWait)) {
             ok = false;
@@ -230,7 +238,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
         __syncwarp();
         if (first && lane == 0) trace_stamp(trace, kTrFirstMmaDone);
         first = false;
-        if (++acc == ACC) {
+        if (++acc == acc_stages) {
           acc = 0;
           acc_phase ^= 1;
         }
@@ -250,7 +258,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
     int acc = 0;
     uint32_t acc_phase = 0;
     uint32_t stg = 0;                       // staging buffers used
-    const uint32_t staging = tiles_base + kSetRingBytes;
+    const uint32_t staging = tiles_base + RING_BYTES;
     bool waited = !epi_defer;               // past the wait for the previous grid
     auto wait_prev = [&]() {
       if (waited) return;
@@ -276,19 +284,21 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
       const bool swap = w.swap != 0;
       const int m0 = c.tm * (swap ? w.mma_n : 128);
       const int n0 = c.tn * (swap ? 128 : w.mma_n);
-      const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(acc * ACC_COLS);
+      const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(acc) * acc_cols;
       // accumulator columns that lie in C (columns of C, or its rows when
       // transposed), and whether any of this warp's accumulator rows do
       const int ncols = swap ? min(w.mma_n, w.m - m0) : min(w.mma_n, w.n - n0);
       const bool live = swap ? n0 + 32 * q < w.n : m0 + 32 * q < w.m;
-      const bool wide = !swap && w.split == 1 && walk.last();   // see go_gemm_kernel
+      // see go_gemm_kernel; the half ring holds 128 rows of 192 fp32 columns
+      const bool wide = !swap && w.split == 1 && walk.last() &&
+                        (CTAS == 1 || ncols * 128 * (OUT_BF16 ? 2 : 4) <= RING_BYTES);
       if (wide) {
         stage_tile_wide<OUT_BF16>(cv, tiles_base, taddr, et, q, m0, ncols);
         wait_prev();
         send_tile_wide<OUT_BF16>(cv, &p.tmap_c[c.g], w.c_tma != 0, tiles_base, et, q, m0, n0, ncols, c.b);
-      } else if (w.split == 1 && !swap) {
+      } else if (CTAS == 1 && w.split == 1 && !swap) {
         wait_prev();
-        store_tile<ACC_COLS, OUT_BF16>(cv, &p.tmap_c[c.g], w.c_tma != 0, staging, stg, taddr, et, q, m0, n0, ncols,
+        store_tile<256, OUT_BF16>(cv, &p.tmap_c[c.g], w.c_tma != 0, staging, stg, taddr, et, q, m0, n0, ncols,
                                        c.b);
       } else {
         wait_prev();
@@ -323,7 +333,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
           mine = *last_flag != 0;
           if (mine) __threadfence();
         }
-        if (mine && w.split > 1 && !swap && w.c_tma == 0) {
+        if (CTAS == 1 && mine && w.split > 1 && !swap && w.c_tma == 0) {
           sum_and_store_tile<OUT_BF16>(cv, tile_parts, tile_f4, w.split, c.s, staging, stg, taddr, et, q, m0, n0,
                                        ncols);
         } else if (mine) {
@@ -351,7 +361,7 @@ __global__ void __launch_bounds__(192, 1) go_gemm_set_kernel(const __grid_consta
       if (first_unit && et == 0) trace_stamp(trace, kTrFirstStore);
       ptx::tc_fence_before();
       ptx::mbar_arrive(ptx::smem_u32(&tempty[acc]));
-      if (++acc == ACC) {
+      if (++acc == acc_stages) {
         acc = 0;
         acc_phase ^= 1;
       }

@@ -146,12 +146,13 @@ const void* kernel_fn_k7(int out_bf16, int fused);
 const void* kernel_fn_k8(int out_bf16, int fused);
 const void* kernel_fn_k9(int out_bf16, int fused);
 const void* kernel_fn_k10(int out_bf16, int fused);
-// The kernel over GEMMs of different single-CTA tile shapes, and its dynamic
-// shared memory: a 192 KB operand ring, two 16 KB staging buffers, 1 KB for
-// alignment, 1 KB for barriers.
-const void* kernel_fn_set(int out_bf16);
-constexpr int kSetRing = 4 * 49152;
-constexpr int kSetSmemBytes = kSetRing + 2 * 16384 + 2048;
+// The kernel over GEMMs of different single-CTA tile shapes, for one or two CTAs
+// per SM, and its dynamic shared memory: a 192 KB operand ring and two 16 KB
+// staging buffers (two CTAs: a 96 KB ring), 1 KB for alignment, 1 KB for
+// barriers.
+const void* kernel_fn_set(int out_bf16, int ctas);
+constexpr int set_ring_bytes(int ctas) { return 4 * 49152 / ctas; }
+constexpr int set_smem_bytes(int ctas) { return set_ring_bytes(ctas) + (ctas == 1 ? 2 * 16384 : 0) + 2048; }
 constexpr int kSetMaxStages = 8;
 
 // Element-wise add (ewise.cu): Z = X + Y over n elements.

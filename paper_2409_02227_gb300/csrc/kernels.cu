@@ -19,10 +19,15 @@ namespace goldy {
 
 #if GOLDY_KIND == 11
 // The kernel over GEMMs of different tile shapes (always the fused form).
-static_assert(kSetRingBytes + 2 * 16384 + 2048 == kSetSmemBytes, "host and kernel agree on the shared memory");
-const void* kernel_fn_set(int out_bf16) {
-  return out_bf16 ? reinterpret_cast<const void*>(&go_gemm_set_kernel<true, kMaxFused>)
-                  : reinterpret_cast<const void*>(&go_gemm_set_kernel<false, kMaxFused>);
+static_assert(kSetRingBytes<1> + 2 * 16384 + 2048 == set_smem_bytes(1) && kSetRingBytes<1> == set_ring_bytes(1) &&
+                  kSetRingBytes<2> + 2048 == set_smem_bytes(2) && kSetRingBytes<2> == set_ring_bytes(2),
+              "host and kernel agree on the shared memory");
+const void* kernel_fn_set(int out_bf16, int ctas) {
+  if (ctas == 2)
+    return out_bf16 ? reinterpret_cast<const void*>(&go_gemm_set_kernel<true, kMaxFused, 2>)
+                    : reinterpret_cast<const void*>(&go_gemm_set_kernel<false, kMaxFused, 2>);
+  return out_bf16 ? reinterpret_cast<const void*>(&go_gemm_set_kernel<true, kMaxFused, 1>)
+                  : reinterpret_cast<const void*>(&go_gemm_set_kernel<false, kMaxFused, 1>);
 }
 #else
 // Inside a template, `if constexpr` discards the other family entirely.

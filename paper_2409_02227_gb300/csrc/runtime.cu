@@ -105,7 +105,7 @@ struct DeviceState {
   int prio_least = 0, prio_greatest = 0;    // cudaDeviceGetStreamPriorityRange
   int* err_word = nullptr;
   int ctas_per_sm[kNumKinds][2][2] = {};   // [kind][bf16 out][fused]; 0 = not yet set up
-  bool set_ready[2] = {};                  // the mixed-shape kernel, set up per output dtype
+  bool set_ready[2][3] = {};               // the mixed-shape kernel, set up per output dtype and CTAs per SM
   int cluster_ok[kNumKinds][2][2][4] = {};  // [..][log2 cluster size]; 0 unknown, 1 yes, -1 no
 };
 
@@ -187,14 +187,14 @@ goldy_status kernel_setup(DeviceState& d, int kind, int out_bf16, int fused, int
   return GOLDY_OK;
 }
 
-// The same for the kernel over GEMMs of different tile shapes (one CTA per SM).
-goldy_status set_kernel_setup(DeviceState& d, int out_bf16) {
+// The same for the kernel over GEMMs of different tile shapes.
+goldy_status set_kernel_setup(DeviceState& d, int out_bf16, int ctas) {
   std::lock_guard<std::mutex> lock(g_mu);
-  if (d.set_ready[out_bf16]) return GOLDY_OK;
-  cudaError_t e =
-      cudaFuncSetAttribute(kernel_fn_set(out_bf16), cudaFuncAttributeMaxDynamicSharedMemorySize, kSetSmemBytes);
+  if (d.set_ready[out_bf16][ctas]) return GOLDY_OK;
+  cudaError_t e = cudaFuncSetAttribute(kernel_fn_set(out_bf16, ctas), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       set_smem_bytes(ctas));
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-  d.set_ready[out_bf16] = true;
+  d.set_ready[out_bf16][ctas] = true;
   return GOLDY_OK;
 }
 
@@ -695,6 +695,24 @@ void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* m
   sh.on = 1;
 }
 
+// CTAs per SM of a launch that mixes tile shapes: two when its units outnumber
+// the SMs (with fewer, a second CTA per SM only halves each unit's ring: 106
+// units 9.7 -> 11.3 us) and it runs with inputs_ready or behind another launch
+// of its run, where the CTAs of consecutive launches overlap (nine GEMMs, 426
+// units: 28.3 -> 19.3 us; 257 units 16.8 -> 9.6; a second launch of 302 units,
+// its run 69.4 -> 57.9).  The kernel for two keeps no staging buffers, so C's
+// rows have to be aligned.
+int set_ctas(const DeviceState& d, const goldy_schedule* s, const int* members, int count, int64_t units,
+             void* const* C) {
+  if (!t_early || units <= sms(d)) return 1;
+  for (int j = 0; j < count; ++j) {
+    const GemmPlan& gp = s->gemms[members[j]];
+    const size_t es = gp.desc.c_dtype == GOLDY_BF16 ? 2 : 4;
+    if (!kKinds[gp.kind].swap_ab && (!aligned(C[members[j]], 16) || size_t(gp.desc.ldc) * es % 16 != 0)) return 1;
+  }
+  return 2;
+}
+
 // One launch over the tiles of `count` (<= kMaxFused) GEMMs of one output
 // dtype: of one kind, or (`mixed`) of any single-CTA kinds through the kernel
 // that reads the tile shape per GEMM.  The grid cap is the sum of the members'
@@ -717,10 +735,10 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   const KindInfo& k = kKinds[kind];
   const bool pair = !mixed && k.pair;
   int ctas = 1;
-  const void* fn = nullptr;
-  goldy_status st = mixed ? set_kernel_setup(d, out_bf16) : kernel_setup(d, kind, out_bf16, 1, &ctas);
+  if (mixed) ctas = set_ctas(d, s, members_in, count, units, C);
+  goldy_status st = mixed ? set_kernel_setup(d, out_bf16, ctas) : kernel_setup(d, kind, out_bf16, 1, &ctas);
   if (st != GOLDY_OK) return st;
-  fn = mixed ? kernel_fn_set(out_bf16) : kernel_fn(kind, out_bf16, 1);
+  const void* fn = mixed ? kernel_fn_set(out_bf16, ctas) : kernel_fn(kind, out_bf16, 1);
   static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
   std::memset(&p, 0, sizeof(p));
   int64_t cap = 0;
@@ -748,6 +766,7 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
     std::stable_sort(members, members + count,
                      [&](int a, int b) { return unit_cost(s->gemms[a]) > unit_cost(s->gemms[b]); });
     deal_units(p.shares, s, members, count, int(pair ? grid / 2 : grid));
+    if (mixed && ctas == 2) p.shares.on = 2;
   }
   units = 0;
   for (int j = 0; j < count; ++j) {
@@ -766,9 +785,10 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   t_stall = 0;
   p.cluster = cluster;
   p.stage_bytes = stage;
-  p.stages = mixed ? std::min(kSetMaxStages, kSetRing / stage) : 0;
+  p.stages = mixed ? std::min(kSetMaxStages, set_ring_bytes(ctas) / stage) : 0;
+  p.acc_stages = stage > stage_bytes(kKinds[2]) ? 1 : 2;   // one 256-column accumulator, or two of 128
   p.trace = trace_for(grid);
-  cudaError_t e = launch_kernel(fn, grid, size_t(mixed ? kSetSmemBytes : smem_bytes(k)), stream, &p, sizeof(p),
+  cudaError_t e = launch_kernel(fn, grid, size_t(mixed ? set_smem_bytes(ctas) : smem_bytes(k)), stream, &p, sizeof(p),
                                 pair ? 2 : cluster);
   if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernel (fused)");
   return GOLDY_OK;

@@ -93,6 +93,12 @@ SETS = {
              (40, 1500, 520, 1, 8, 1), (130, 200, 72, 1, 2, 2), (20, 70, 264, 1, 6, 1)],
     # strided batches next to plain GEMMs; many more units than CTAs; K shorter than a block
     "batched": [(130, 136, 200, 6, 2, 1), (40, 72, 64, 9, 8, 1), (1500, 1100, 136, 1, 0, 1), (300, 300, 8, 1, 3, 1)],
+    # more units than SMs and aligned rows: with inputs_ready two CTAs per SM, with one 256-column accumulator ...
+    "two_per_sm_wide": [(520, 4096, 456, 1, 4, 1), (200, 2048, 2056, 1, 2, 4), (33, 2048, 520, 1, 8, 2),
+                        (20, 1032, 4104, 1, 6, 8), (300, 72, 72, 1, 0, 1), (600, 520, 1032, 1, 4, 2)],
+    # ... and with two of 128
+    "two_per_sm": [(200, 2048, 2056, 1, 2, 4), (33, 4096, 520, 1, 8, 2), (20, 1032, 4104, 1, 6, 8),
+                   (300, 72, 72, 1, 0, 1), (1100, 1048, 200, 1, 2, 1), (64, 2048, 64, 1, 9, 1)],
     # one unit per GEMM: fewer units than CTAs
     "tiny": [(1, 1, 8, 1, 0, 1), (16, 64, 64, 1, 8, 1), (5, 130, 16, 1, 2, 1)],
 }
