@@ -5,6 +5,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -170,6 +171,17 @@ const void* ewise_kernel_fn(int bf16);
 
 }  // namespace goldy
 
+namespace goldy {
+// The shares of one launch (see assign_units), kept with the plan: they follow
+// from the launch's GEMMs and its bins alone.
+struct DealtUnits {
+  std::vector<int> members;
+  int bins = 0;
+  std::vector<uint16_t> rounds, first;
+};
+constexpr size_t kMaxDealt = 16;   // launches kept per plan (two per run, for each grid size seen)
+}  // namespace goldy
+
 struct goldy_schedule {
   int flags = 0;
   bool auto_plan = false;   // planned by GOLDY_PLAN_AUTO (fused: one launch per kernel family, see run_impl)
@@ -178,6 +190,8 @@ struct goldy_schedule {
   std::vector<goldy::GemmPlan> gemms;
   std::vector<goldy::Group> groups;
   goldy::Runtime* rt = nullptr;   // created on first goldy_run
+  mutable std::mutex dealt_mu;    // guards dealt
+  mutable std::vector<goldy::DealtUnits> dealt;
 };
 
 // A GEMM co-scheduled with an element-wise add (planner.cpp builds it,

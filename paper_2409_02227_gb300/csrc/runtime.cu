@@ -670,10 +670,23 @@ double unit_cost(const GemmPlan& gp) {
 
 // Equal shares of a launch's units for its `bins` CTAs (pairs); `members`
 // sorted by descending unit cost.  Left off (round-robin) when the table
-// cannot hold them.
+// cannot hold them.  Computed once per plan, launch and grid (about 1.3 us per
+// GEMM, of a goldy_run of 16 us for six).
 void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* members, int count, int bins) {
   sh.on = 0;
   if (count < 2 || bins > kMaxBins) return;
+  auto copy = [&](const DealtUnits& d) {
+    std::copy(d.rounds.begin(), d.rounds.end(), sh.rounds);
+    for (int j = 0; j < count; ++j)
+      std::copy_n(d.first.begin() + int64_t(j) * (bins + 1), bins + 1, sh.first[j]);
+    sh.on = 1;
+  };
+  {
+    std::lock_guard<std::mutex> lock(s->dealt_mu);
+    for (const DealtUnits& d : s->dealt)
+      if (d.bins == bins && d.members.size() == size_t(count) && std::equal(members, members + count, d.members.begin()))
+        return copy(d);
+  }
   int64_t units[kMaxFused];
   double cost[kMaxFused];
   bool rotate[kMaxFused];
@@ -686,13 +699,16 @@ void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* m
     cost[j] = unit_cost(s->gemms[members[j]]);
     if (units[j] > 65535) return;
   }
-  static thread_local int32_t first[kMaxFused * (kMaxBins + 1)];
-  int32_t rounds[kMaxFused];
+  int32_t first[kMaxFused * (kMaxBins + 1)], rounds[kMaxFused];
   assign_units(count, units, cost, rotate, bins, rounds, first);
-  for (int j = 0; j < count; ++j) sh.rounds[j] = uint16_t(rounds[j]);
-  for (int j = 0; j < count; ++j)
-    for (int b = 0; b <= bins; ++b) sh.first[j][b] = uint16_t(first[j * (bins + 1) + b]);
-  sh.on = 1;
+  DealtUnits d;
+  d.members.assign(members, members + count);
+  d.bins = bins;
+  d.rounds.assign(rounds, rounds + count);
+  d.first.assign(first, first + int64_t(count) * (bins + 1));
+  copy(d);
+  std::lock_guard<std::mutex> lock(s->dealt_mu);
+  if (s->dealt.size() < kMaxDealt) s->dealt.push_back(std::move(d));
 }
 
 // CTAs per SM of a launch that mixes tile shapes: two when its units outnumber
