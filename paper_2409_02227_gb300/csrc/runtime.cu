@@ -578,11 +578,12 @@ unsigned long long* trace_for(unsigned grid) {
 // therefore takes the two-per-SM kind of the same tile shape (same K split,
 // same order of sums: the same bytes), so that a run no longer starts when the
 // one before leaves its SMs.  Measured back to back: four layers of eight 32 x
-// 4096 x 1024 59.1 -> 45.7 us, of four 128 x 1024 x 4096 split 4 41.6 -> 36.1
-// us, 753 x 1152 x 704 and a smaller one 6.6 -> 4.4 us.  A launch whose splits
-// reduce in clusters only when two runs do not fit side by side anyway: the
+// 4096 x 1024 59.6 -> 47.7 us, of four 128 x 1024 x 4096 split 4 41.8 -> 36.3
+// us, 753 x 1152 x 704 and a smaller one 6.7 -> 4.5 us, two 18 x 3904 x 896 3.5
+// -> 2.6 us.  K splits only when two runs do not fit side by side anyway: the
 // two-per-SM kinds have no room for pushed partials (two 256 x 256 x 512 split
-// 4, 64 CTAs: 3.06 -> 3.90 us).  256-wide tiles keep their deeper ring.
+// 4, 64 CTAs: 3.06 -> 3.90 us), and 39 units of 31 K blocks lost 10%.  256-wide
+// tiles keep their deeper ring.
 int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, int split) {
   if (!t_early || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 || kKinds[kind].mma_n > 128) return kind;
   const int twin = kind + 1;
@@ -592,9 +593,10 @@ int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, i
                     kKinds[9].ctas_per_sm == 2,
                 "a full kind is followed by the half kind of its tile shape");
   if (units > 2 * int64_t(sms(d))) return kind;
-  int ctas = 0;   // (the set-up also readies the kernel for the cluster query)
-  if (kernel_setup(d, twin, out_bf16, fused, &ctas) != GOLDY_OK || ctas < 2) return kind;
-  if (split > 1 && (2 * units <= sms(d) || !cluster_feasible(d, twin, out_bf16, fused, split))) return kind;
+  int ctas = 0;   // the set-up readies the kernel for the cluster query
+  if (kernel_setup(d, twin, out_bf16, fused, &ctas) != GOLDY_OK) return kind;
+  if (split != 1 && 2 * units <= sms(d)) return kind;
+  if (split > 1 && !cluster_feasible(d, twin, out_bf16, fused, split)) return kind;
   return twin;
 }
 
@@ -609,6 +611,7 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
   int ctas = 0;
   goldy_status st = kernel_setup(d, kind, out_bf16, 0, &ctas);
   if (st != GOLDY_OK) return st;
+  if (kind != gp.kind) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
   if (gp.units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one GEMM");
 
   LaunchParams<1> p;
@@ -754,6 +757,7 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   if (mixed) ctas = set_ctas(d, s, members_in, count, units, C);
   goldy_status st = mixed ? set_kernel_setup(d, out_bf16, ctas) : kernel_setup(d, kind, out_bf16, 1, &ctas);
   if (st != GOLDY_OK) return st;
+  if (kind != g0.kind) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
   const void* fn = mixed ? kernel_fn_set(out_bf16, ctas) : kernel_fn(kind, out_bf16, 1);
   static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
   std::memset(&p, 0, sizeof(p));
