@@ -391,12 +391,35 @@ goldy_status encode_3d(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t
 
 bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
-// One GEMM's slot of a launch: tensor maps and work description.
-template <int MAXG>
-goldy_status fill_slot(LaunchParams<MAXG>& p, int j, const GemmPlan& gp, const void* A, const void* B, void* C,
-                       uint8_t* ws, int32_t unit_begin) {
-  const goldy_gemm_desc& g = gp.desc;
+// The kind whose tile shape computes a GEMM planned for gp.kind.  A 128 x 128
+// tile over at most 32 rows (or 64) is computed transposed, 128 columns by 32
+// (64) rows: the same tiles and K splits, each element the same sum in the same
+// order, without the padded rows' shared-memory fill and MMA work, and with all
+// four epilogue warps at the rows there are.  Eight 32 x 4096 x 1024 18.5 ->
+// 16.2 us, two 20 x 1024 x 4096 split 4 11.3 -> 9.6, eight 17 x 6144 x 512 15.6
+// -> 13.8.  With 33 to 64 rows the transposed stores cost more, so only where K
+// splits (64 x 512 x 8192 split 8 11.5 -> 10.2) or the main loop is long (33 x
+// 4096 x 8192 23.5 -> 22.0; but 64 x 8192 x 1024 9.2 -> 9.8).
+int shape_kind(const GemmPlan& gp) {
   const KindInfo& k = kKinds[gp.kind];
+  if (k.pair || k.swap_ab || k.mma_n != 128) return gp.kind;
+  constexpr int kN128 = 2, kT32 = 6, kT64 = 8;        // each followed by its two-per-SM kind
+  static_assert(kKinds[kN128].mma_n == 128 && kKinds[kT32].mma_n == 32 && kKinds[kT32].swap_ab == 1 &&
+                    kKinds[kT64].mma_n == 64 && kKinds[kT64].swap_ab == 1 && kKinds[kN128 + 1].mma_n == 128 &&
+                    kKinds[kT32 + 1].mma_n == 32 && kKinds[kT64 + 1].mma_n == 64,
+                "kind order");
+  if (gp.desc.M <= 32) return gp.kind - kN128 + kT32;
+  if (gp.desc.M <= 64 && (gp.split > 1 || gp.k_blocks >= 32)) return gp.kind - kN128 + kT64;
+  return gp.kind;
+}
+
+// One GEMM's slot of a launch: tensor maps and work description, for the tile
+// shape of `kind`.
+template <int MAXG>
+goldy_status fill_slot(LaunchParams<MAXG>& p, int j, const GemmPlan& gp, int kind, const void* A, const void* B,
+                       void* C, uint8_t* ws, int32_t unit_begin) {
+  const goldy_gemm_desc& g = gp.desc;
+  const KindInfo& k = kKinds[kind];
   // batch strides in bytes; a single GEMM gets the packed stride (never read)
   const bool batched = g.batch > 1;
   const uint64_t sa = uint64_t(batched ? g.stride_a : g.M * g.lda) * 2;
@@ -606,17 +629,18 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
                          cudaStream_t stream, double scale = 0.0) {
   if (degenerate(gp)) return launch_degenerate(gp, C, stream);
   const int out_bf16 = gp.desc.c_dtype == GOLDY_BF16 ? 1 : 0;
-  const int kind = run_kind(d, gp.kind, out_bf16, 0, gp.units, gp.split);
+  const int planned = shape_kind(gp);
+  const int kind = run_kind(d, planned, out_bf16, 0, gp.units, gp.split);
   const KindInfo& k = kKinds[kind];
   int ctas = 0;
   goldy_status st = kernel_setup(d, kind, out_bf16, 0, &ctas);
   if (st != GOLDY_OK) return st;
-  if (kind != gp.kind) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
+  if (kind != planned) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
   if (gp.units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one GEMM");
 
   LaunchParams<1> p;
   std::memset(&p, 0, sizeof(p));
-  st = fill_slot(p, 0, gp, A, B, C, ws, 0);
+  st = fill_slot(p, 0, gp, kind, A, B, C, ws, 0);
   if (st != GOLDY_OK) return st;
   p.n_gemms = 1;
   p.total_units = int32_t(gp.units);
@@ -656,7 +680,7 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
 // bytes/ns, a tile leaves at about 45 bytes/ns (each SM's share of the memory
 // rate).  Only the ratios matter.
 double unit_cost(const GemmPlan& gp) {
-  const KindInfo& k = kKinds[gp.kind];
+  const KindInfo& k = kKinds[shape_kind(gp)];
   const goldy_gemm_desc& g = gp.desc;
   const double rows = double(g.M) / double(gp.tiles_m), cols = double(g.N) / double(gp.tiles_n);
   const double kb = double(gp.k_blocks) / double(gp.split);
@@ -727,7 +751,7 @@ int set_ctas(const DeviceState& d, const goldy_schedule* s, const int* members, 
   for (int j = 0; j < count; ++j) {
     const GemmPlan& gp = s->gemms[members[j]];
     const size_t es = gp.desc.c_dtype == GOLDY_BF16 ? 2 : 4;
-    if (!kKinds[gp.kind].swap_ab && (!aligned(C[members[j]], 16) || size_t(gp.desc.ldc) * es % 16 != 0)) return 1;
+    if (!kKinds[shape_kind(gp)].swap_ab && (!aligned(C[members[j]], 16) || size_t(gp.desc.ldc) * es % 16 != 0)) return 1;
   }
   return 2;
 }
@@ -750,14 +774,19 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
     units += s->gemms[members_in[j]].units;
     if (s->gemms[members_in[j]].split != split) split = 0;
   }
-  const int kind = mixed ? g0.kind : run_kind(d, g0.kind, out_bf16, 1, units, split);
+  // one tile shape for the launch: the planned kind's, or the transposed one
+  // that suits all of its GEMMs; a mixed launch takes each GEMM's own
+  int planned = shape_kind(g0);
+  for (int j = 1; j < count && !mixed; ++j)
+    if (shape_kind(s->gemms[members_in[j]]) != planned) planned = g0.kind;
+  const int kind = mixed ? planned : run_kind(d, planned, out_bf16, 1, units, split);
   const KindInfo& k = kKinds[kind];
   const bool pair = !mixed && k.pair;
   int ctas = 1;
   if (mixed) ctas = set_ctas(d, s, members_in, count, units, C);
   goldy_status st = mixed ? set_kernel_setup(d, out_bf16, ctas) : kernel_setup(d, kind, out_bf16, 1, &ctas);
   if (st != GOLDY_OK) return st;
-  if (kind != g0.kind) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
+  if (kind != planned) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
   const void* fn = mixed ? kernel_fn_set(out_bf16, ctas) : kernel_fn(kind, out_bf16, 1);
   static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
   std::memset(&p, 0, sizeof(p));
@@ -766,7 +795,7 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   for (int j = 0; j < count; ++j) {
     const GemmPlan& gp = s->gemms[members_in[j]];
     cap += std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(gp.variant).rc_div);
-    stage = std::max(stage, stage_bytes(kKinds[gp.kind]));
+    stage = std::max(stage, stage_bytes(kKinds[mixed ? shape_kind(gp) : kind]));
   }
   if (units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one launch");
   if (scale > 0.0) cap = std::max<int64_t>(1, int64_t(double(cap) * scale));
@@ -791,7 +820,8 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   units = 0;
   for (int j = 0; j < count; ++j) {
     const GemmPlan& gp = s->gemms[members[j]];
-    st = fill_slot(p, j, gp, A[members[j]], B[members[j]], C[members[j]], ws, int32_t(units));
+    st = fill_slot(p, j, gp, mixed ? shape_kind(gp) : kind, A[members[j]], B[members[j]], C[members[j]], ws,
+                   int32_t(units));
     if (st != GOLDY_OK) return st;
     units += gp.units;
   }
