@@ -607,8 +607,14 @@ unsigned long long* trace_for(unsigned grid) {
 // two-per-SM kinds have no room for pushed partials (two 256 x 256 x 512 split
 // 4, 64 CTAs: 3.06 -> 3.90 us), and 39 units of 31 K blocks lost 10%.  256-wide
 // tiles keep their deeper ring.
+//
+// Without inputs_ready the same kind pays where one CTA per SM would leave a
+// second round for a few units: between one and two units per SM all of them
+// run at once (four layers of eight 32 x 4096 x 1024, 256 units: 64.5 -> 59.5
+// us; 777 x 1501 x 1003, 168 units: 12.6 -> 10.7; two 89 x 960 x 1984 split:
+// 14.5 -> 8.6).
 int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, int split) {
-  if (!t_early || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 || kKinds[kind].mma_n > 128) return kind;
+  if ((!t_early && units <= sms(d)) || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 || kKinds[kind].mma_n > 128) return kind;
   const int twin = kind + 1;
   static_assert(kKinds[1].mma_n == kKinds[0].mma_n && kKinds[3].mma_n == kKinds[2].mma_n &&
                     kKinds[7].mma_n == kKinds[6].mma_n && kKinds[9].mma_n == kKinds[8].mma_n &&
