@@ -7,8 +7,10 @@
 // most CD GEMMs are in flight, each stream running its GEMMs back to back),
 // and joins back into streams[0] before the next group starts.  In the fused
 // launch mode the GEMMs of a wave that share a kernel kind go out as one
-// persistent launch over all their tiles instead.  The whole run can be
-// captured once into a CUDA graph and replayed with one launch.
+// persistent launch over all their tiles instead, and a plan of the dynamic
+// logic as at most two launches (per output dtype) over the tiles of all its
+// GEMMs.  The whole run can be captured once into a CUDA graph and replayed
+// with one launch.
 //
 // Per GEMM the host encodes two TMA tensor maps (A and B), sizes the
 // persistent grid as min(units, resident CTAs per SM * SMs / rc_div) — the
@@ -750,13 +752,19 @@ void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* m
 // of its run, where the CTAs of consecutive launches overlap (nine GEMMs, 426
 // units: 28.3 -> 19.3 us; 257 units 16.8 -> 9.6; a second launch of 302 units,
 // its run 69.4 -> 57.9).  The kernel for two keeps no staging buffers, so C's
-// rows have to be aligned.
+// rows have to be aligned.  One, too, where 256-column tiles write f32: there
+// is room for one accumulator that wide, so each tile's MMAs wait for the
+// 128 KB that the tile before stores from registers (sets of 8 to 14 GEMMs with
+// f32 C and 225 to 1428 units: two per SM 22.8, 34.8, 76, 92, 110, 134 us, one
+// 17.0, 19.6, 54, 72, 77, 104; with bf16 C two stay faster, 9.6 against 17.1
+// and 64.7 against 70.3).
 int set_ctas(const DeviceState& d, const goldy_schedule* s, const int* members, int count, int64_t units,
              void* const* C) {
   if (!t_early || units <= sms(d)) return 1;
   for (int j = 0; j < count; ++j) {
     const GemmPlan& gp = s->gemms[members[j]];
     const size_t es = gp.desc.c_dtype == GOLDY_BF16 ? 2 : 4;
+    if (es == 4 && stage_bytes(kKinds[shape_kind(gp)]) > stage_bytes(kKinds[2])) return 1;
     if (!kKinds[shape_kind(gp)].swap_ab && (!aligned(C[members[j]], 16) || size_t(gp.desc.ldc) * es % 16 != 0)) return 1;
   }
   return 2;
