@@ -189,7 +189,8 @@ def peaks():
         return 6800.0, 1900.0, 1700.0, "fallback"
 
 
-KERNEL_SOURCES = ("go_kernel.cuh", "go_kernel_pair.cuh", "sm103_ptx.cuh", "kernels.cu", "goldy_internal.h")
+KERNEL_SOURCES = ("go_kernel.cuh", "go_kernel_pair.cuh", "go_kernel_set.cuh", "sm103_ptx.cuh", "kernels.cu",
+                  "goldy_internal.h")
 
 
 def csrc_hash() -> str:
