@@ -607,8 +607,10 @@ unsigned long long* trace_for(unsigned grid) {
 // us, 753 x 1152 x 704 and a smaller one 6.7 -> 4.5 us, two 18 x 3904 x 896 3.5
 // -> 2.6 us.  K splits only when two runs do not fit side by side anyway: the
 // two-per-SM kinds have no room for pushed partials (two 256 x 256 x 512 split
-// 4, 64 CTAs: 3.06 -> 3.90 us), and 39 units of 31 K blocks lost 10%.  256-wide
-// tiles keep their deeper ring.
+// 4, 64 CTAs: 3.06 -> 3.90 us), and 39 units of 31 K blocks lost 10%.  GEMMs of
+// different splits (split = 0) only with more units than SMs: 86 units of four
+// GEMMs 8.3 us on the two-per-SM kind, 6.6 on the planned one.  256-wide tiles
+// keep their deeper ring.
 //
 // Without inputs_ready the same kind pays where one CTA per SM would leave a
 // second round for a few units: between one and two units per SM all of them
@@ -627,6 +629,7 @@ int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, i
   int ctas = 0;   // the set-up readies the kernel for the cluster query
   if (kernel_setup(d, twin, out_bf16, fused, &ctas) != GOLDY_OK) return kind;
   if (split != 1 && 2 * units <= sms(d)) return kind;
+  if (split == 0 && units <= sms(d)) return kind;
   if (split > 1 && !cluster_feasible(d, twin, out_bf16, fused, split)) return kind;
   return twin;
 }
