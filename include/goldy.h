@@ -409,10 +409,9 @@ goldy_status goldy_corun_plan(const goldy_gemm_desc* gemm, const goldy_ewise_des
  * variant; the add's grid-cap divisor; device workspace bytes (split-K). */
 goldy_status goldy_corun_query(const goldy_corun* c, int* concurrent, int* gemm_variant, int* add_rc_div,
                                size_t* workspace_bytes);
-/* Enqueue on streams[0]: the GEMM C = A B and the add, at once when concurrent
- * (the add starts as soon as the work before the co-run is complete and ends
- * after the GEMM; streams[1] is asked for but not used), else the add after
- * the GEMM.  X, Y, Z: device arrays of n elements; the vector path
+/* Enqueue: the GEMM C = A B on streams[0]; the add on streams[1] (forked
+ * from and joined back into streams[0]) when concurrent, else on streams[0]
+ * after the GEMM.  X, Y, Z: device arrays of n elements; the vector path
  * needs them 16-byte aligned (others take a scalar path).  Asynchronous. */
 goldy_status goldy_corun_run(const goldy_corun* c, const void* A, const void* B, void* C, void* workspace,
                              size_t workspace_bytes, const void* X, const void* Y, void* Z, void* const* streams,

@@ -9,10 +9,6 @@
 // Arithmetic: IEEE fp32 addition with round-to-nearest-even; bf16 inputs are
 // widened exactly and the fp32 sum is rounded to bf16 (RNE).  Pointers that
 // are not 16-byte aligned take the scalar path for the whole array.
-//
-// Next to a GEMM it may run "beside" it: a programmatic dependent launch on the
-// GEMM's own stream that starts once the GEMM's CTAs are all past their wait
-// for the work before (LaunchParams::late_trigger) and ends after the GEMM.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -56,8 +52,6 @@ __global__ void __launch_bounds__(kEwiseThreads) ewise_add_kernel(const EwisePar
   void* __restrict__ z = p.z;
   const int64_t n = p.n;
   const int vec_ok = p.vec_ok;
-  // beside the kernel before: the next kernel on the stream may set up now
-  if (p.beside) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int kPerVec = BF16 ? 8 : 4;
   const int64_t stride = int64_t(gridDim.x) * kEwiseThreads;
   const int64_t tid = int64_t(blockIdx.x) * kEwiseThreads + threadIdx.x;
@@ -94,9 +88,6 @@ __global__ void __launch_bounds__(kEwiseThreads) ewise_add_kernel(const EwisePar
       static_cast<float*>(z)[i] = __fadd_rn(static_cast<const float*>(x)[i], static_cast<const float*>(y)[i]);
     }
   }
-  // beside the kernel before: this grid ends after it, so that whatever waits
-  // for this grid has waited for both
-  if (p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace

@@ -163,7 +163,7 @@ struct EwiseParams {
   void* z;
   int64_t n;
   int32_t vec_ok;   // all three pointers 16-byte aligned
-  int32_t beside;   // 1: launched beside the kernel before it on the stream (see ewise.cu)
+  int32_t pad;
 };
 constexpr int kEwiseThreads = 256;
 constexpr int kEwiseCtasPerSm = 8;
@@ -202,6 +202,7 @@ struct goldy_corun {
   int policy = 0;
   int concurrent = 0;
   int add_rc_div = 1;
+  goldy::Runtime* rt = nullptr;     // fork/join events, created on first run
 };
 
 namespace goldy {

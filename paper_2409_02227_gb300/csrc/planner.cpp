@@ -802,5 +802,6 @@ extern "C" goldy_status goldy_corun_query(const goldy_corun* c, int* concurrent,
 extern "C" void goldy_corun_free(goldy_corun* c) {
   if (!c) return;
   goldy_schedule_free(c->gemm);
+  goldy::runtime_release(c->rt);
   delete c;
 }

@@ -267,8 +267,8 @@ cudaError_t launch_kernel(const void* fn, unsigned grid, size_t smem, cudaStream
 
 // A kernel with `block` threads per CTA and no cluster (recorded like launch_kernel).
 cudaError_t launch_kernel_threads(const void* fn, unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
-                                  const void* params, size_t params_size, bool pdl) {
-  if (!t_rec) return launch_kernel_now(fn, grid, smem, stream, const_cast<void*>(params), 0, block, pdl);
+                                  const void* params, size_t params_size) {
+  if (!t_rec) return launch_kernel_now(fn, grid, smem, stream, const_cast<void*>(params), 0, block);
   Op op;
   op.kind = Op::kKernel;
   op.stream = stream;
@@ -276,7 +276,6 @@ cudaError_t launch_kernel_threads(const void* fn, unsigned grid, unsigned block,
   op.grid = grid;
   op.block = block;
   op.smem = smem;
-  op.pdl = pdl;
   op.params.resize((params_size + 7) / 8);
   std::memcpy(op.params.data(), params, params_size);
   t_rec->push_back(std::move(op));
@@ -921,7 +920,7 @@ struct RunOptionsReset {
 // recorded run owns its events), otherwise the schedule's are used.
 static goldy_status run_impl(const goldy_schedule* s, const void* const* A, const void* const* B, void* const* C,
                              void* workspace, size_t workspace_bytes, void* const* streams, int n_streams,
-                             const goldy_run_opts* opts, Runtime* own_rt, bool late_trigger = false) {
+                             const goldy_run_opts* opts, Runtime* own_rt) {
   if (!s || !A || !B || !C || !streams) return fail(GOLDY_ERR_INVALID_ARG, "null argument");
   if (n_streams < s->max_streams) return fail(GOLDY_ERR_INVALID_ARG, "fewer streams than the schedule needs");
   if (s->workspace_bytes > 0) {
@@ -971,7 +970,6 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   t_early = (opts && opts->inputs_ready) ? 1 : 0;
   t_wait_ns = opts ? uint64_t(opts->wait_limit_us) * 1000ull : 0;
   t_stall = (opts && opts->test_stall_first_stage) ? 1 : 0;
-  t_late = late_trigger ? 1 : 0;
   auto hook = [&](void* const* evs, const int* members, int n, cudaStream_t stream) -> goldy_status {
     if (!evs) return GOLDY_OK;
     for (int j = 0; j < n; ++j) {
@@ -1326,6 +1324,7 @@ extern "C" goldy_status goldy_run_ex(const goldy_schedule* s, const void* const*
 struct goldy_exec {
   std::vector<Op> ops;
   Runtime* rt = nullptr;
+  Runtime* rt2 = nullptr;    // a co-run's own fork/join events
   CUcontext ctx = nullptr;   // the partition's context to make current while replaying (null: none)
   cudaStream_t main = nullptr;
 };
@@ -1420,6 +1419,7 @@ extern "C" goldy_status goldy_exec_time(const goldy_exec* const* execs, int n, i
 extern "C" void goldy_exec_free(goldy_exec* x) {
   if (!x) return;
   runtime_release(x->rt);
+  runtime_release(x->rt2);
   delete x;
 }
 
@@ -1427,7 +1427,7 @@ extern "C" void goldy_exec_free(goldy_exec* x) {
 // Element-wise add and a GEMM co-scheduled with it
 // ---------------------------------------------------------------------------
 static goldy_status launch_ewise(const DeviceState& d, const goldy_ewise_desc& ew, const void* X, const void* Y,
-                                 void* Z, int rc_div, cudaStream_t stream, bool beside = false) {
+                                 void* Z, int rc_div, cudaStream_t stream) {
   if (ew.n == 0) return GOLDY_OK;
   EwiseParams p;
   std::memset(&p, 0, sizeof(p));
@@ -1436,13 +1436,12 @@ static goldy_status launch_ewise(const DeviceState& d, const goldy_ewise_desc& e
   p.z = Z;
   p.n = ew.n;
   p.vec_ok = (aligned(X, 16) && aligned(Y, 16) && aligned(Z, 16)) ? 1 : 0;
-  p.beside = beside ? 1 : 0;
   const int64_t per_vec = ew.dtype == GOLDY_BF16 ? 8 : 4;
   const int64_t work = p.vec_ok ? (ew.n + per_vec - 1) / per_vec : ew.n;
   const int64_t cap = std::max<int64_t>(1, int64_t(kEwiseCtasPerSm) * sms(d) / rc_div);
   const unsigned grid = unsigned(std::max<int64_t>(1, std::min<int64_t>(cap, (work + kEwiseThreads - 1) / kEwiseThreads)));
   cudaError_t e = launch_kernel_threads(ewise_kernel_fn(ew.dtype == GOLDY_BF16 ? 1 : 0), grid, kEwiseThreads, 0,
-                                        stream, &p, sizeof(p), beside);
+                                        stream, &p, sizeof(p));
   if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernel (element-wise add)");
   return GOLDY_OK;
 }
@@ -1473,9 +1472,10 @@ extern "C" goldy_status goldy_ewise_add(const void* X, const void* Y, void* Z, i
 }
 
 // gemm_rt: events of the GEMM's run (null: the GEMM schedule's own);
+// corun_rt: the fork/join events of the two streams (null: the co-run's own).
 static goldy_status corun_impl(const goldy_corun* c, const void* A, const void* B, void* C, void* ws,
                                size_t ws_bytes, const void* X, const void* Y, void* Z, void* const* streams,
-                               int n_streams, Runtime* gemm_rt) {
+                               int n_streams, Runtime* gemm_rt, Runtime* corun_rt) {
   if (!c || !streams) return fail(GOLDY_ERR_INVALID_ARG, "null argument");
   if (n_streams < (c->concurrent ? 2 : 1)) return fail(GOLDY_ERR_INVALID_ARG, "fewer streams than the co-run needs");
   goldy_status st = check_ewise(c->ew, X, Y, Z, c->add_rc_div);
@@ -1496,22 +1496,39 @@ static goldy_status corun_impl(const goldy_corun* c, const void* A, const void* 
     st = launch_ewise(*d, c->ew, X, Y, Z, c->add_rc_div, s0);
     return st == GOLDY_OK ? ok() : st;
   }
-  // At once on streams[0] alone: the GEMM's CTAs let the add start when they
-  // are past their wait for the work before the co-run, and the add ends after
-  // the GEMM.  (On a second stream, forked and joined by events, the same pair
-  // of 1024 x 4096 x 1024 bf16 and its add took 18.4 us; so it takes 16.3.)  Without a GEMM
-  // kernel there is nothing to start beside: the add follows in stream order.
-  const bool beside = !degenerate(c->gemm->gemms[0]);
-  st = run_impl(c->gemm, a, b, cc, ws, ws_bytes, streams, 1, nullptr, gemm_rt, beside);
+  Runtime* rt = corun_rt;
+  if (!rt) {
+    goldy_corun* mc = const_cast<goldy_corun*>(c);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (mc->rt && (mc->rt->device != dev || mc->rt->green != part.green())) {
+      runtime_release(mc->rt);
+      mc->rt = nullptr;
+    }
+    if (!mc->rt) {
+      mc->rt = new_runtime(dev, part.green(), &st);
+      if (!mc->rt) return st;
+    }
+    rt = mc->rt;
+  }
+  cudaStream_t s1 = static_cast<cudaStream_t>(streams[1]);
+  cudaError_t e = enq_event_record(rt->fork, s0);
+  if (e == cudaSuccess) e = enq_wait(s1, rt->fork);
+  if (e != cudaSuccess) return cuda_fail(e, "co-run fork");
+  st = run_impl(c->gemm, a, b, cc, ws, ws_bytes, streams, 1, nullptr, gemm_rt);
   if (st != GOLDY_OK) return st;
-  st = launch_ewise(*d, c->ew, X, Y, Z, c->add_rc_div, s0, beside);
-  return st == GOLDY_OK ? ok() : st;
+  st = launch_ewise(*d, c->ew, X, Y, Z, c->add_rc_div, s1);
+  if (st != GOLDY_OK) return st;
+  e = enq_event_record(rt->join[0], s1);
+  if (e == cudaSuccess) e = enq_wait(s0, rt->join[0]);
+  if (e != cudaSuccess) return cuda_fail(e, "co-run join");
+  return ok();
 }
 
 extern "C" goldy_status goldy_corun_run(const goldy_corun* c, const void* A, const void* B, void* C, void* workspace,
                                         size_t workspace_bytes, const void* X, const void* Y, void* Z,
                                         void* const* streams, int n_streams) {
-  return corun_impl(c, A, B, C, workspace, workspace_bytes, X, Y, Z, streams, n_streams, nullptr);
+  return corun_impl(c, A, B, C, workspace, workspace_bytes, X, Y, Z, streams, n_streams, nullptr, nullptr);
 }
 
 extern "C" goldy_status goldy_corun_exec_create(const goldy_corun* c, const void* A, const void* B, void* C,
@@ -1534,12 +1551,13 @@ extern "C" goldy_status goldy_corun_exec_create(const goldy_corun* c, const void
   }
   x->main = static_cast<cudaStream_t>(streams[0]);
   x->rt = new_runtime(dev, part.green(), &st);
-  if (!x->rt) {
+  if (x->rt) x->rt2 = new_runtime(dev, part.green(), &st);
+  if (!x->rt || !x->rt2) {
     goldy_exec_free(x);
     return st;
   }
   t_rec = &x->ops;
-  st = corun_impl(c, A, B, C, workspace, workspace_bytes, X, Y, Z, streams, n_streams, x->rt);
+  st = corun_impl(c, A, B, C, workspace, workspace_bytes, X, Y, Z, streams, n_streams, x->rt, x->rt2);
   t_rec = nullptr;
   if (st != GOLDY_OK) {
     std::string why = goldy_last_error();
