@@ -106,11 +106,14 @@ typedef struct goldy_graph goldy_graph;
  * of all other kinds' (per output dtype, at most 16 GEMMs per launch), their
  * tiles dealt out to the GPU's CTAs in equal shares, longest first; both go
  * out on streams[0] alone, the largest first, each overlapping the previous
- * one's tail (no fork, no join).  FUSED otherwise (explicit schedules, the
- * forced policies), and for a plan of a single launch: within each group, the
- * GEMMs of a wave that share a kernel kind and output dtype go into ONE
- * persistent launch over the concatenation of their tiles (at most 16 GEMMs
- * per launch); its grid cap is the sum of the members' caps.  A wave's
+ * one's tail.  Without inputs_ready such a run starts after what was enqueued
+ * before it on the streams that the waves' own launches would have used, and
+ * what is enqueued there later starts after the run.  FUSED otherwise
+ * (explicit schedules, the forced policies), and for a plan of a single
+ * launch: within each group, the GEMMs of a wave that share a kernel kind and
+ * output dtype go into ONE persistent launch over the concatenation of their
+ * tiles (at most 16 GEMMs per launch); its grid cap is the sum of the members'
+ * caps.  A wave's
  * launches carry launch priorities ranked by their FLOPs, and the first wave's
  * largest launch goes out first (outside a stream capture the other streams
  * also wait until all of its CTAs have begun).  Groups are not separated by a

@@ -73,10 +73,12 @@ struct Op {
   void* ptr = nullptr;
   size_t pitch = 0, width = 0, height = 0;
   cudaEvent_t ev = nullptr;
+  bool capture_only = false;         // replayed only while streams[0] is being captured
 };
 
 namespace {
 thread_local std::vector<Op>* t_rec = nullptr;   // non-null: record instead of enqueue
+thread_local bool t_capture_only = false;        // Op::capture_only of what is recorded next
 // GO-Kernel launches carry a programmatic dependency on the previous kernel of
 // their stream (the kernels wait for it before touching global memory) unless
 // the run asks for serial launches
@@ -307,6 +309,7 @@ cudaError_t enq_event_record(cudaEvent_t ev, cudaStream_t stream, bool external 
   op.kind = external ? Op::kEventRecordExternal : Op::kEventRecord;
   op.stream = stream;
   op.ev = ev;
+  op.capture_only = t_capture_only;
   t_rec->push_back(std::move(op));
   return cudaSuccess;
 }
@@ -317,6 +320,7 @@ cudaError_t enq_wait(cudaStream_t stream, cudaEvent_t ev) {
   op.kind = Op::kWait;
   op.stream = stream;
   op.ev = ev;
+  op.capture_only = t_capture_only;
   t_rec->push_back(std::move(op));
   return cudaSuccess;
 }
@@ -1039,7 +1043,10 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // already is one launch stays as it is: its kind's own kernel is the better
   // one there (deeper ring, split-K in a cluster).  Explicit schedules and the
   // forced policies keep one launch per wave and kind.
-  if (fused && s->auto_plan && sets.size() > 1) {
+  uint32_t slots = 0;                        // the slots on whose streams these launches would go out
+  for (const LaunchSet& ls : sets) slots |= 1u << ls.slot;
+  const bool join_launches = fused && s->auto_plan && sets.size() > 1;
+  if (join_launches) {
     std::vector<LaunchSet> joined;
     joined.reserve(sets.size());
     int singles[2] = {0, 0};               // launches of single-CTA kinds per output dtype
@@ -1256,6 +1263,28 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       if (sets[a].wave != sets[b].wave) return sets[a].wave < sets[b].wave;
       return sets[a].rank < sets[b].rank;
     });
+  // A joined run without inputs_ready keeps the order of the streams that its
+  // launches would have gone out on each by itself: it starts after what the
+  // caller enqueued there before, and what is enqueued there later starts after
+  // it.  (Within a stream capture the streams are first brought into the
+  // capture and joined again at the end.)  The events cost what the forks and
+  // joins of separate launches do: runs back to back with one side stream 27.2
+  // -> 31.2 us (five GEMMs of odd sizes), with two 16.1 -> 19.0 (six GEMMs).
+  uint32_t ordered = 0;
+  if (join_launches && !t_early)
+    for (int k = 1; k < GOLDY_MAX_STREAMS; ++k)
+      if ((slots >> k & 1) && streams[k] != streams[0]) ordered |= 1u << k;
+  const bool in_capture = capturing != cudaStreamCaptureStatusNone;
+  auto capture_only = [&](auto&& what, uint32_t side) -> goldy_status {
+    if (!in_capture && !t_rec) return GOLDY_OK;
+    t_capture_only = true;
+    const goldy_status r = what(side);
+    t_capture_only = false;
+    return r;
+  };
+  st = capture_only(fork, ordered);
+  if (st == GOLDY_OK) st = join(ordered);
+  if (st != GOLDY_OK) return st;
   const bool pdl = t_pdl;
   int last_group[GOLDY_MAX_STREAMS];
   bool waited[GOLDY_MAX_STREAMS];
@@ -1312,6 +1341,9 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
     if (st != GOLDY_OK) return st;
     t0 = t1;
   }
+  st = fork(ordered);
+  if (st == GOLDY_OK) st = capture_only(join, ordered);
+  if (st != GOLDY_OK) return st;
   return ok();
 }
 
@@ -1323,6 +1355,7 @@ extern "C" goldy_status goldy_run_ex(const goldy_schedule* s, const void* const*
 
 struct goldy_exec {
   std::vector<Op> ops;
+  bool capture_ops = false;  // any of them for captures only
   Runtime* rt = nullptr;
   Runtime* rt2 = nullptr;    // a co-run's own fork/join events
   CUcontext ctx = nullptr;   // the partition's context to make current while replaying (null: none)
@@ -1357,6 +1390,7 @@ extern "C" goldy_status goldy_exec_create(const goldy_schedule* s, const void* c
   t_rec = &x->ops;
   st = run_impl(s, A, B, C, workspace, workspace_bytes, streams, n_streams, opts, x->rt);
   t_rec = nullptr;
+  for (const Op& op : x->ops) x->capture_ops = x->capture_ops || op.capture_only;
   if (st != GOLDY_OK) {
     std::string why = goldy_last_error();
     runtime_release(x->rt);
@@ -1371,9 +1405,12 @@ extern "C" goldy_status goldy_exec_launch(const goldy_exec* x) {
   if (!x) return fail(GOLDY_ERR_INVALID_ARG, "null exec");
   if (x->ctx && green_api().push(x->ctx) != CUDA_SUCCESS) return fail(GOLDY_ERR_CUDA, "cuCtxPushCurrent failed");
   cudaError_t e = cudaSuccess;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (x->capture_ops) e = cudaStreamIsCapturing(x->main, &capturing);
   for (const Op& op : x->ops) {
-    e = replay(op);
     if (e != cudaSuccess) break;
+    if (op.capture_only && capturing == cudaStreamCaptureStatusNone) continue;
+    e = replay(op);
   }
   if (x->ctx) {
     CUcontext popped = nullptr;
@@ -1396,11 +1433,11 @@ extern "C" goldy_status goldy_exec_time(const goldy_exec* const* execs, int n, i
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   for (int k = 0; k < warmup && e == cudaSuccess; ++k)
     for (const Op& op : execs[k % n]->ops)
-      if ((e = replay(op)) != cudaSuccess) break;
+      if (!op.capture_only && (e = replay(op)) != cudaSuccess) break;
   if (e == cudaSuccess) e = cudaEventRecord(e0, x0->main);
   for (int k = 0; k < reps && e == cudaSuccess; ++k)
     for (const Op& op : execs[k % n]->ops)
-      if ((e = replay(op)) != cudaSuccess) break;
+      if (!op.capture_only && (e = replay(op)) != cudaSuccess) break;
   if (e == cudaSuccess) e = cudaEventRecord(e1, x0->main);
   if (e == cudaSuccess) e = cudaEventSynchronize(e1);
   float ms = 0.f;

@@ -5,6 +5,7 @@ import pytest
 import torch
 
 from paper_2409_02227_gb300 import goldy as G
+from paper_2409_02227_gb300 import profile_lut as P
 
 pytestmark = pytest.mark.gpu
 
@@ -49,4 +50,80 @@ def test_coruns_add_keeps_the_order_of_its_stream(cuda_ok, policy, prepared):
     for x, o in zip(src, out):
         assert torch.equal(o, x + Y)
     assert torch.equal(C.float(), (A.double() @ B.double()).bfloat16().float())
+    del ex
+
+
+# (M, N, K, kind): one launch each of a fused wave, so one stream each; the
+# first set's three kinds join into two launches, the second's into one
+WAVES = [[(100, 320, 1496, 2), (40, 1500, 1200, 8), (700, 600, 1096, 10)],
+         [(200, 320, 456, 2), (40, 300, 520, 8), (20, 600, 1000, 6)]]
+
+
+@pytest.mark.parametrize("how", ["run", "exec", "captured run", "captured exec"])
+@pytest.mark.parametrize("wave", [0, 1])
+def test_joined_run_keeps_the_order_of_its_streams(cuda_ok, wave, how):
+    specs = WAVES[wave]
+    entries, descs = [], []
+    for M, N, K, kind in specs:
+        d = G.desc(M, N, K, F32, lda=K, ldb=(N + 7) // 8 * 8, ldc=N)
+        key = G.goldy_bucket_key(d)
+        entries.append((((key >> 24) & 255, (key >> 16) & 255, (key >> 8) & 255, key & 255), 4,
+                        [G.variant_id(kind, 1, 1)] * 5))
+        descs.append(d)
+    lut = G.goldy_lut_from_memory(P.write_lut(entries, G.goldy_variant_count(), 152))
+    plan = G.goldy_plan(descs, lut, G.GOLDY_PLAN_AUTO | G.GOLDY_PLAN_FUSED)
+    slots = [G.goldy_schedule_entry(plan, i)[2] for i in range(len(specs))]
+    assert sorted(slots) == [0, 1, 2]
+    _, _, n_streams, ws_bytes = G.goldy_schedule_query(plan)
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    new = lambda r, c: torch.randint(-3, 4, (r, c), generator=gen, device="cuda").bfloat16()
+    src = [[new(M, K) for M, N, K, _ in specs] for _ in range(3)]
+    A = [torch.zeros_like(a) for a in src[0]]
+    B = [new(K, (N + 7) // 8 * 8) for M, N, K, _ in specs]
+    C = [torch.zeros((M, N), device="cuda") for M, N, K, _ in specs]
+    out = [[torch.zeros_like(c) for c in C] for _ in src]
+    ws = torch.zeros(max(ws_bytes, 256), dtype=torch.uint8, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(n_streams)]
+    handles = [s.cuda_stream for s in streams]
+    args = (plan, [a.data_ptr() for a in A], [b.data_ptr() for b in B], [c.data_ptr() for c in C], ws.data_ptr(),
+            ws_bytes, handles)
+    ex = G.goldy_exec_create(*args) if "exec" in how else None
+    launch = (lambda: G.goldy_exec_launch(ex)) if ex else (lambda: G.goldy_run(*args))
+
+    def step(a, o):
+        # each GEMM's A is written, and its C read, on the stream of its slot
+        for i, k in enumerate(slots):
+            _late(streams[k], A[i], a[i])
+        launch()
+        for i, k in enumerate(slots):
+            with torch.cuda.stream(streams[k]):
+                o[i].copy_(C[i])
+
+    torch.cuda.synchronize()
+    if "captured" in how:
+        launch()                              # loads the kernels
+        torch.cuda.synchronize()
+        for a, o in zip(src, out):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=streams[0]):
+                for s in streams[1:]:
+                    s.wait_stream(streams[0])
+                step(a, o)
+                for s in streams[1:]:
+                    streams[0].wait_stream(s)
+            g.replay()
+            torch.cuda.synchronize()
+        # a capture that uses streams[0] alone: the run leaves no stream unjoined
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=streams[0]):
+            launch()
+        g.replay()
+    else:
+        for a, o in zip(src, out):
+            step(a, o)
+    torch.cuda.synchronize()
+    assert G.goldy_device_error(clear=True) == 0
+    for a, o in zip(src, out):
+        for i, (M, N, K, _) in enumerate(specs):
+            assert torch.equal(o[i].double(), a[i].double() @ B[i][:, :N].double()), (specs[i], how)
     del ex
