@@ -145,7 +145,12 @@ const char* goldy_last_error(void);
  * or a quarter of it (Sec. 4.2.1's GPU, GPU/2, GPU/4).  With a split S > 1
  * the S K-ranges of a tile are summed in split order 0 .. S-1 (in a cluster
  * of S CTAs, or by the last split to arrive, through the workspace; a CTA-pair
- * kind always through the workspace). */
+ * kind always through the workspace).  An explicit schedule
+ * (goldy_schedule_build) runs exactly the kinds its variants name.  A planned
+ * GEMM (goldy_plan, goldy_corun_plan) or goldy_gemm_noalloc may run on another
+ * kind where that is faster: the transposed tile of the same size for few rows
+ * of C, or the two-CTAs-per-SM kind of the same tile, with the variant's K
+ * split and the same order of sums, so the same bytes. */
 typedef struct goldy_variant_info {
   int32_t id;
   int32_t kind;           /* tile/footprint family, 0 .. n_kinds-1 */
@@ -249,7 +254,8 @@ goldy_status goldy_plan_ex(const goldy_gemm_desc* descs, int n, const goldy_lut*
  * increasing order, ids 0 .. n_groups-1 all used), with variant
  * variant_of[i], on stream slot slot_of[i] (< GOLDY_MAX_STREAMS).  A group's
  * CD is its number of distinct slots.  flags: 0 or GOLDY_PLAN_FUSED (waves are
- * then the group's members taken CD at a time, in GEMM index order). */
+ * then the group's members taken CD at a time, in GEMM index order).  Launches
+ * run the kinds that the variants name. */
 goldy_status goldy_schedule_build(const goldy_gemm_desc* descs, int n, const int* group_of,
                                   const int* variant_of, const int* slot_of, int flags,
                                   goldy_schedule** out);

@@ -185,6 +185,7 @@ constexpr size_t kMaxDealt = 16;   // launches kept per plan (two per run, for e
 struct goldy_schedule {
   int flags = 0;
   bool auto_plan = false;   // planned by GOLDY_PLAN_AUTO (fused: one launch per kernel family, see run_impl)
+  bool named_variants = false;   // goldy_schedule_build: launches run exactly the kinds named
   int max_streams = 1;
   size_t workspace_bytes = 0;
   std::vector<goldy::GemmPlan> gemms;

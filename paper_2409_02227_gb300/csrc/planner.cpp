@@ -627,6 +627,7 @@ extern "C" goldy_status goldy_schedule_build(const goldy_gemm_desc* descs, int n
   goldy_status st = new_schedule(descs, n, &s);
   if (st != GOLDY_OK) return st;
   s->flags = flags;
+  s->named_variants = true;
   int n_groups = 0;
   for (int i = 0; i < n; ++i) {
     if (group_of[i] < 0 || group_of[i] >= n || variant_of[i] < 0 || variant_of[i] >= kNumVariants ||
@@ -775,6 +776,7 @@ extern "C" goldy_status goldy_corun_plan(const goldy_gemm_desc* gemm, const gold
   goldy_schedule* s = nullptr;
   st = goldy_schedule_build(gemm, 1, &group, &variant, &slot, 0, &s);
   if (st != GOLDY_OK) return st;
+  s->named_variants = false;         // planned, like goldy_plan's
   goldy_corun* c = new (std::nothrow) goldy_corun();
   if (!c) {
     goldy_schedule_free(s);

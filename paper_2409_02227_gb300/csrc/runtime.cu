@@ -87,6 +87,7 @@ thread_local bool t_pdl = true;
 // early operand loads, the bounded-wait limit, and the test stall hook
 // (first launch of the run only).
 thread_local int32_t t_early = 0;
+thread_local bool t_named = false;  // an explicit schedule: its launches run the kinds it names
 thread_local int32_t t_late = 0;    // LaunchParams::late_trigger of the next launch
 thread_local uint64_t t_wait_ns = 0;
 thread_local int32_t t_stall = 0;
@@ -396,7 +397,8 @@ goldy_status encode_3d(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t
 
 bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
-// The kind whose tile shape computes a GEMM planned for gp.kind.  A 128 x 128
+// The kind whose tile shape computes a GEMM planned for gp.kind (an explicit
+// schedule measures the kinds it names: there gp.kind itself).  A 128 x 128
 // tile over at most 32 rows (or 64) is computed transposed, 128 columns by 32
 // (64) rows: the same tiles and K splits, each element the same sum in the same
 // order, without the padded rows' shared-memory fill and MMA work, and with all
@@ -407,7 +409,7 @@ bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) %
 // 4096 x 8192 23.5 -> 22.0; but 64 x 8192 x 1024 9.2 -> 9.8).
 int shape_kind(const GemmPlan& gp) {
   const KindInfo& k = kKinds[gp.kind];
-  if (k.pair || k.swap_ab || k.mma_n != 128) return gp.kind;
+  if (t_named || k.pair || k.swap_ab || k.mma_n != 128) return gp.kind;
   constexpr int kN128 = 2, kT32 = 6, kT64 = 8;        // each followed by its two-per-SM kind
   static_assert(kKinds[kN128].mma_n == 128 && kKinds[kT32].mma_n == 32 && kKinds[kT32].swap_ab == 1 &&
                     kKinds[kT64].mma_n == 64 && kKinds[kT64].swap_ab == 1 && kKinds[kN128 + 1].mma_n == 128 &&
@@ -600,7 +602,8 @@ unsigned long long* trace_for(unsigned grid) {
   return region;
 }
 
-// The kind that runs a launch planned for `kind`.  With inputs_ready the next
+// The kind that runs a launch planned for `kind` (an explicit schedule runs
+// the kinds it names).  With inputs_ready the next
 // run's CTAs may load and multiply while this run's wait for their stores, if
 // an SM has room for them: a launch of at most two CTAs' worth of units per SM
 // therefore takes the two-per-SM kind of the same tile shape (same K split,
@@ -621,7 +624,7 @@ unsigned long long* trace_for(unsigned grid) {
 // us; 777 x 1501 x 1003, 168 units: 12.6 -> 10.7; two 89 x 960 x 1984 split:
 // 14.5 -> 8.6).
 int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, int split) {
-  if ((!t_early && units <= sms(d)) || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 || kKinds[kind].mma_n > 128) return kind;
+  if (t_named || (!t_early && units <= sms(d)) || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 || kKinds[kind].mma_n > 128) return kind;
   const int twin = kind + 1;
   static_assert(kKinds[1].mma_n == kKinds[0].mma_n && kKinds[3].mma_n == kKinds[2].mma_n &&
                     kKinds[7].mma_n == kKinds[6].mma_n && kKinds[9].mma_n == kKinds[8].mma_n &&
@@ -913,6 +916,7 @@ struct RunOptionsReset {
     t_trace_used = 0;
     t_pdl = true;
     t_early = 0;
+    t_named = false;
     t_late = 0;
     t_wait_ns = 0;
     t_stall = 0;
@@ -972,6 +976,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   t_trace_used = 0;
   t_pdl = !(opts && opts->serial_launch);
   t_early = (opts && opts->inputs_ready) ? 1 : 0;
+  t_named = s->named_variants;
   t_wait_ns = opts ? uint64_t(opts->wait_limit_us) * 1000ull : 0;
   t_stall = (opts && opts->test_stall_first_stage) ? 1 : 0;
   auto hook = [&](void* const* evs, const int* members, int n, cudaStream_t stream) -> goldy_status {
