@@ -623,15 +623,23 @@ unsigned long long* trace_for(unsigned grid) {
 // run at once (four layers of eight 32 x 4096 x 1024, 256 units: 64.5 -> 59.5
 // us; 777 x 1501 x 1003, 168 units: 12.6 -> 10.7; two 89 x 960 x 1984 split:
 // 14.5 -> 8.6).
-int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, int split) {
-  if (t_named || (!t_early && units <= sms(d)) || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 || kKinds[kind].mma_n > 128) return kind;
+//
+// `cap` is the planned kind's grid cap.  A launch that may not use the whole GPU
+// keeps its share: it takes the two-per-SM kind only where the cap does not bind
+// (so that its grid is the same, of CTAs half the size), never to run a second
+// round's units on more SMs than it was given.
+int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, int split, int64_t cap) {
+  const bool whole = cap >= sms(d);
+  if (t_named || (!t_early && (!whole || units <= sms(d))) || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 ||
+      kKinds[kind].mma_n > 128)
+    return kind;
   const int twin = kind + 1;
   static_assert(kKinds[1].mma_n == kKinds[0].mma_n && kKinds[3].mma_n == kKinds[2].mma_n &&
                     kKinds[7].mma_n == kKinds[6].mma_n && kKinds[9].mma_n == kKinds[8].mma_n &&
                     kKinds[1].ctas_per_sm == 2 && kKinds[3].ctas_per_sm == 2 && kKinds[7].ctas_per_sm == 2 &&
                     kKinds[9].ctas_per_sm == 2,
                 "a full kind is followed by the half kind of its tile shape");
-  if (units > 2 * int64_t(sms(d))) return kind;
+  if (units > (whole ? 2 * int64_t(sms(d)) : cap)) return kind;
   int ctas = 0;   // the set-up readies the kernel for the cluster query
   if (kernel_setup(d, twin, out_bf16, fused, &ctas) != GOLDY_OK) return kind;
   if (split != 1 && 2 * units <= sms(d)) return kind;
@@ -647,12 +655,14 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
   if (degenerate(gp)) return launch_degenerate(gp, C, stream);
   const int out_bf16 = gp.desc.c_dtype == GOLDY_BF16 ? 1 : 0;
   const int planned = shape_kind(gp);
-  const int kind = run_kind(d, planned, out_bf16, 0, gp.units, gp.split);
-  const KindInfo& k = kKinds[kind];
   int ctas = 0;
-  goldy_status st = kernel_setup(d, kind, out_bf16, 0, &ctas);
+  goldy_status st = kernel_setup(d, planned, out_bf16, 0, &ctas);
   if (st != GOLDY_OK) return st;
-  if (kind != planned) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
+  int64_t cap = std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(gp.variant).rc_div);
+  if (scale > 0.0) cap = std::min<int64_t>(int64_t(ctas) * sms(d), std::max<int64_t>(1, int64_t(double(cap) * scale)));
+  const int kind = run_kind(d, planned, out_bf16, 0, gp.units, gp.split, cap);
+  if (kind != planned && cap >= sms(d)) cap = 2 * int64_t(sms(d));
+  const KindInfo& k = kKinds[kind];
   if (gp.units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one GEMM");
 
   LaunchParams<1> p;
@@ -668,9 +678,6 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
   p.stall_test = t_stall;
   t_stall = 0;
 
-  const Variant v = variant_of(gp.variant);
-  int64_t cap = std::max<int64_t>(1, int64_t(ctas) * sms(d) / v.rc_div);
-  if (scale > 0.0) cap = std::min<int64_t>(int64_t(ctas) * sms(d), std::max<int64_t>(1, int64_t(double(cap) * scale)));
   if (k.pair) {
     const unsigned grid = pair_grid(gp.units, cap);
     p.trace = trace_for(grid);
@@ -802,27 +809,26 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   int planned = shape_kind(g0);
   for (int j = 1; j < count && !mixed; ++j)
     if (shape_kind(s->gemms[members_in[j]]) != planned) planned = g0.kind;
-  const int kind = mixed ? planned : run_kind(d, planned, out_bf16, 1, units, split);
-  const KindInfo& k = kKinds[kind];
-  const bool pair = !mixed && k.pair;
+  const bool pair = !mixed && kKinds[planned].pair;
   int ctas = 1;
   if (mixed) ctas = set_ctas(d, s, members_in, count, units, C);
-  goldy_status st = mixed ? set_kernel_setup(d, out_bf16, ctas) : kernel_setup(d, kind, out_bf16, 1, &ctas);
+  goldy_status st = mixed ? set_kernel_setup(d, out_bf16, ctas) : kernel_setup(d, planned, out_bf16, 1, &ctas);
   if (st != GOLDY_OK) return st;
-  if (kind != planned) ctas = 2;   // (see run_kind: room for twice the planned kind's CTAs)
+  if (units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one launch");
+  int64_t cap = 0;
+  for (int j = 0; j < count; ++j)
+    cap += std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(s->gemms[members_in[j]].variant).rc_div);
+  if (scale > 0.0) cap = std::max<int64_t>(1, int64_t(double(cap) * scale));
+  cap = whole ? int64_t(ctas) * sms(d) : std::min<int64_t>(cap, int64_t(ctas) * sms(d));
+  const int kind = mixed ? planned : run_kind(d, planned, out_bf16, 1, units, split, cap);
+  if (kind != planned && cap >= sms(d)) cap = 2 * int64_t(sms(d));
+  const KindInfo& k = kKinds[kind];
   const void* fn = mixed ? kernel_fn_set(out_bf16, ctas) : kernel_fn(kind, out_bf16, 1);
   static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
   std::memset(&p, 0, sizeof(p));
-  int64_t cap = 0;
   int stage = 0;
-  for (int j = 0; j < count; ++j) {
-    const GemmPlan& gp = s->gemms[members_in[j]];
-    cap += std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(gp.variant).rc_div);
-    stage = std::max(stage, stage_bytes(kKinds[mixed ? shape_kind(gp) : kind]));
-  }
-  if (units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one launch");
-  if (scale > 0.0) cap = std::max<int64_t>(1, int64_t(double(cap) * scale));
-  cap = whole ? int64_t(ctas) * sms(d) : std::min<int64_t>(cap, int64_t(ctas) * sms(d));
+  for (int j = 0; j < count; ++j)
+    stage = std::max(stage, stage_bytes(kKinds[mixed ? shape_kind(s->gemms[members_in[j]]) : kind]));
   const int cluster =
       (!mixed && !pair && split > 1 && cluster_feasible(d, kind, out_bf16, 1, split)) ? split : 0;
   const unsigned grid = pair ? pair_grid(units, cap) : launch_grid(units, cap, cluster);
