@@ -110,7 +110,9 @@ struct DeviceState {
   int prio_least = 0, prio_greatest = 0;    // cudaDeviceGetStreamPriorityRange
   int* err_word = nullptr;
   int ctas_per_sm[kNumKinds][2][2] = {};   // [kind][bf16 out][fused]; 0 = not yet set up
-  bool set_ready[2][3] = {};               // the mixed-shape kernel, set up per output dtype and CTAs per SM
+  int two_fit[kNumKinds][2][2] = {};       // two CTAs on an SM (see two_per_sm): 0 unknown, 1 yes, -1 no
+  int set_ready[2][3] = {};                // the mixed-shape kernel per output dtype and CTAs per SM: 0 not yet set
+                                           // up, 1 set up, -1 that many CTAs do not fit on an SM
   int cluster_ok[kNumKinds][2][2][4] = {};  // [..][log2 cluster size]; 0 unknown, 1 yes, -1 no
 };
 
@@ -192,14 +194,49 @@ goldy_status kernel_setup(DeviceState& d, int kind, int out_bf16, int fused, int
   return GOLDY_OK;
 }
 
-// The same for the kernel over GEMMs of different tile shapes.
-goldy_status set_kernel_setup(DeviceState& d, int out_bf16, int ctas) {
+// Do two CTAs of this kernel fit on an SM?  The occupancy query cannot say: it
+// rounds a CTA's six warps up to two per SM partition, and answers one CTA for
+// every kernel of more than 128 registers a thread.  The partitions take the
+// warps of two CTAs in turn, three each, which fit at up to 168 registers (that
+// is what the kernels' launch bounds hold them to; 304 CTAs of 152 SMs do start
+// at once).
+bool two_per_sm(const void* fn, int smem) {
+  cudaFuncAttributes a;
+  int dev = 0, regs = 0, sm_bytes = 0, reserved = 0;
+  if (cudaFuncGetAttributes(&a, fn) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  constexpr int kWarpsPerPartition = 2 * (kThreads / 32) / 4;
+  const int per_warp = (a.numRegs * 32 + 255) / 256 * 256;
+  return kWarpsPerPartition * per_warp <= regs / 4 && 2 * (smem + int(a.sharedSizeBytes) + reserved) <= sm_bytes;
+}
+
+// The same for a kind's kernel (set up before); tensor memory of the two-per-SM
+// kinds is at most half an SM's.
+bool two_per_sm(DeviceState& d, int kind, int out_bf16, int fused) {
   std::lock_guard<std::mutex> lock(g_mu);
-  if (d.set_ready[out_bf16][ctas]) return GOLDY_OK;
-  cudaError_t e = cudaFuncSetAttribute(kernel_fn_set(out_bf16, ctas), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       set_smem_bytes(ctas));
-  if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-  d.set_ready[out_bf16][ctas] = true;
+  int& t = d.two_fit[kind][out_bf16][fused];
+  if (t == 0)
+    t = tmem_cols(kKinds[kind]) <= 256 && two_per_sm(kernel_fn(kind, out_bf16, fused), smem_bytes(kKinds[kind])) ? 1 : -1;
+  return t > 0;
+}
+
+// Sets up the kernel over GEMMs of different tile shapes for `ctas` CTAs per
+// SM; false in *fits when they do not fit.
+goldy_status set_kernel_setup(DeviceState& d, int out_bf16, int ctas, bool* fits) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  int& ready = d.set_ready[out_bf16][ctas];
+  if (ready == 0) {
+    const void* fn = kernel_fn_set(out_bf16, ctas);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, set_smem_bytes(ctas));
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+    ready = ctas == 1 || two_per_sm(fn, set_smem_bytes(ctas)) ? 1 : -1;
+  }
+  *fits = ready > 0;
   return GOLDY_OK;
 }
 
@@ -641,7 +678,7 @@ int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, i
                 "a full kind is followed by the half kind of its tile shape");
   if (units > (whole ? 2 * int64_t(sms(d)) : cap)) return kind;
   int ctas = 0;   // the set-up readies the kernel for the cluster query
-  if (kernel_setup(d, twin, out_bf16, fused, &ctas) != GOLDY_OK) return kind;
+  if (kernel_setup(d, twin, out_bf16, fused, &ctas) != GOLDY_OK || !two_per_sm(d, twin, out_bf16, fused)) return kind;
   if (split != 1 && 2 * units <= sms(d)) return kind;
   if (split == 0 && units <= sms(d)) return kind;
   if (split > 1 && !cluster_feasible(d, twin, out_bf16, fused, split)) return kind;
@@ -811,8 +848,11 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
     if (shape_kind(s->gemms[members_in[j]]) != planned) planned = g0.kind;
   const bool pair = !mixed && kKinds[planned].pair;
   int ctas = 1;
+  bool fits = true;
   if (mixed) ctas = set_ctas(d, s, members_in, count, units, C);
-  goldy_status st = mixed ? set_kernel_setup(d, out_bf16, ctas) : kernel_setup(d, planned, out_bf16, 1, &ctas);
+  goldy_status st =
+      mixed ? set_kernel_setup(d, out_bf16, ctas, &fits) : kernel_setup(d, planned, out_bf16, 1, &ctas);
+  if (st == GOLDY_OK && !fits) st = set_kernel_setup(d, out_bf16, ctas = 1, &fits);
   if (st != GOLDY_OK) return st;
   if (units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one launch");
   int64_t cap = 0;

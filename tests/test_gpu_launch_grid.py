@@ -60,3 +60,49 @@ def test_fused_launch_keeps_the_sum_of_its_shares(cuda_ok, ready):
         units = 2 * tiles
         want = units if cap >= sms and units <= 2 * sms else min(units, cap)
         assert _run(_plan(shapes, [2, 2], rc, G.GOLDY_PLAN_FUSED), shapes, inputs_ready=ready) == [want]
+
+
+def _all_at_once(plan, shapes, out, grid, **opts):
+    """Whether one launch of `grid` CTAs has all of them running at one time (operands of zeros)."""
+    _, _, n_streams, ws_bytes = G.goldy_schedule_query(plan)
+    dt = torch.bfloat16 if out == BF16 else torch.float32
+    A = [torch.zeros((M, K), dtype=torch.bfloat16, device="cuda") for M, N, K in shapes]
+    B = [torch.zeros((K, N), dtype=torch.bfloat16, device="cuda") for M, N, K in shapes]
+    C = [torch.empty((M, N), dtype=dt, device="cuda") for M, N, K in shapes]
+    ws = torch.zeros(max(ws_bytes, 256), dtype=torch.uint8, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(n_streams)]
+    trace = torch.zeros(1024 * 16, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(2):                       # the first run loads the kernel
+        G.goldy_run_ex(plan, [t.data_ptr() for t in A], [t.data_ptr() for t in B], [t.data_ptr() for t in C],
+                       ws.data_ptr(), ws_bytes, [s.cuda_stream for s in streams], trace=trace.data_ptr(),
+                       trace_ctas=1024, **opts)
+        torch.cuda.synchronize()
+    assert G.goldy_device_error(clear=True) == 0
+    rows = trace.view(1024, 16).cpu()
+    rows = rows[rows[:, 0] != 0]
+    assert rows.shape[0] == grid and set(rows[:, 12].tolist()) == {grid}
+    return int(rows[:, 0].max()) < int(rows[:, 9].min())
+
+
+@pytest.mark.parametrize("out", [F32, BF16])
+@pytest.mark.parametrize("kind,M,tile_cols", [(0, 100, 64), (2, 100, 128), (6, 30, 128), (8, 60, 128)])
+def test_two_ctas_per_sm_are_resident(cuda_ok, kind, M, tile_cols, out):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shapes = [(M, 2 * sms * tile_cols, 4096)]
+    for flags in (0, G.GOLDY_PLAN_FUSED):
+        assert _all_at_once(_plan(shapes, [kind], 1, flags, out), shapes, out, 2 * sms)
+
+
+@pytest.mark.parametrize("out", [F32, BF16])
+@pytest.mark.parametrize("wide", [False, True])
+def test_mixed_launch_has_two_ctas_per_sm(cuda_ok, wide, out):
+    # two kinds in one launch of two units per SM; one CTA per SM where 256-column tiles write f32
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    kind, cols = (4, 256) if wide else (2, 128)
+    shapes = [(200, sms // 2 * cols, 4096), (60, sms * 128, 8192)]
+    plan = _plan(shapes, [kind, 8], 1, G.GOLDY_PLAN_FUSED, out)
+    kinds = [G.goldy_variant_info_get(G.goldy_schedule_entry(plan, i)[1])["kind"] for i in range(2)]
+    assert kinds == [kind, 8]
+    one = wide and out == F32
+    assert _all_at_once(plan, shapes, out, sms if one else 2 * sms, inputs_ready=True)
