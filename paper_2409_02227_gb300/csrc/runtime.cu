@@ -1049,41 +1049,45 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
     int members[kMaxFused];
   };
   std::vector<LaunchSet> sets;
-  sets.reserve(s->gemms.size());
-  for (size_t g = 0; g < s->groups.size(); ++g) {
-    const Group& grp = s->groups[g];
-    const int size = int(grp.members.size());
-    const int wave = fused ? std::max(1, grp.cd) : 1;
-    for (int w0 = 0; w0 < size; w0 += wave) {
-      const size_t first_set = sets.size();
-      for (int j = w0; j < std::min(size, w0 + wave); ++j) {
-        const int i = grp.members[j];
-        const GemmPlan& gp = s->gemms[i];
-        size_t target = sets.size();
-        if (fused && !degenerate(gp))
-          for (size_t t = first_set; t < sets.size(); ++t) {
-            const GemmPlan& g0 = s->gemms[sets[t].members[0]];
-            if (!sets[t].degenerate && sets[t].n < kMaxFused && g0.kind == gp.kind &&
-                g0.desc.c_dtype == gp.desc.c_dtype) {
-              target = t;
-              break;
+  // by_split: a launch's GEMMs also have one K split (so that clusters reduce it)
+  auto make_sets = [&](std::vector<LaunchSet>& sets, bool by_split) {
+    sets.reserve(s->gemms.size());
+    for (size_t g = 0; g < s->groups.size(); ++g) {
+      const Group& grp = s->groups[g];
+      const int size = int(grp.members.size());
+      const int wave = fused ? std::max(1, grp.cd) : 1;
+      for (int w0 = 0; w0 < size; w0 += wave) {
+        const size_t first_set = sets.size();
+        for (int j = w0; j < std::min(size, w0 + wave); ++j) {
+          const int i = grp.members[j];
+          const GemmPlan& gp = s->gemms[i];
+          size_t target = sets.size();
+          if (fused && !degenerate(gp))
+            for (size_t t = first_set; t < sets.size(); ++t) {
+              const GemmPlan& g0 = s->gemms[sets[t].members[0]];
+              if (!sets[t].degenerate && sets[t].n < kMaxFused && g0.kind == gp.kind &&
+                  g0.desc.c_dtype == gp.desc.c_dtype && (!by_split || g0.split == gp.split)) {
+                target = t;
+                break;
+              }
             }
+          if (target == sets.size()) {
+            LaunchSet ls{};
+            ls.group = int(g);
+            ls.slot = gp.slot;
+            ls.degenerate = degenerate(gp) ? 1 : 0;
+            ls.wave = w0;
+            ls.prio = kNoPriority;
+            sets.push_back(ls);
           }
-        if (target == sets.size()) {
-          LaunchSet ls{};
-          ls.group = int(g);
-          ls.slot = gp.slot;
-          ls.degenerate = degenerate(gp) ? 1 : 0;
-          ls.wave = w0;
-          ls.prio = kNoPriority;
-          sets.push_back(ls);
+          sets[target].members[sets[target].n++] = i;
+          sets[target].flops += 2.0 * double(gp.desc.M) * double(gp.desc.N) * double(gp.desc.K) *
+                                double(std::max<int64_t>(1, gp.desc.batch));
         }
-        sets[target].members[sets[target].n++] = i;
-        sets[target].flops += 2.0 * double(gp.desc.M) * double(gp.desc.N) * double(gp.desc.K) *
-                              double(std::max<int64_t>(1, gp.desc.batch));
       }
     }
-  }
+  };
+  make_sets(sets, false);
   // Fused plans of the dynamic logic: the launches of all waves and groups
   // join into one launch of the pair kernel and one of the kernel over
   // different single-CTA tile shapes (per output dtype, at most kMaxFused
@@ -1094,9 +1098,35 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // already is one launch stays as it is: its kind's own kernel is the better
   // one there (deeper ring, split-K in a cluster).  Explicit schedules and the
   // forced policies keep one launch per wave and kind.
+  //
+  // Two launches stay apart where most of the work is K splits that clusters
+  // reduce on chip and all units fit on the GPU at once: joined, their partials
+  // go through the workspace (written, counted, read back), which costs more
+  // than the one start saved.  With inputs_ready, 38 x 704 x 256 next to 122 x
+  // 1536 x 2624 split 4 (bf16) 9.4 -> 5.4 us; 22 x 704 x 256 next to 262 x 896 x 1344
+  // split 4 9.8 -> 7.3; 58 x 960 x 384 next to 33 x 320 x 640 split 8 (f32) 6.2 -> 4.5.
+  // At least two thirds of the units, split 4 or more: with half of them split
+  // (22 x 896 x 320 next to 24 x 384 x 320 split 5) apart is slower, 5.5 -> 7.2,
+  // and a split of 2 (38 of 47 units) exchanges too little, 4.8 -> 5.2.
   uint32_t slots = 0;                        // the slots on whose streams these launches would go out
   for (const LaunchSet& ls : sets) slots |= 1u << ls.slot;
-  const bool join_launches = fused && s->auto_plan && sets.size() > 1;
+  bool apart = false;
+  if (fused && s->auto_plan) {
+    int64_t units = 0, reducible = 0;
+    bool single = true;                      // single-CTA kinds only, nothing degenerate
+    for (const GemmPlan& gp : s->gemms) {
+      single = single && !degenerate(gp) && !kKinds[gp.kind].pair;
+      units += gp.units;
+      if (gp.split >= 4) reducible += gp.units;
+    }
+    if (single && units <= sms(*d) && 3 * reducible >= 2 * units) {
+      std::vector<LaunchSet> by_split;
+      make_sets(by_split, true);
+      apart = by_split.size() == 2;
+      if (apart) sets.swap(by_split);
+    }
+  }
+  const bool join_launches = fused && s->auto_plan && !apart && sets.size() > 1;
   if (join_launches) {
     std::vector<LaunchSet> joined;
     joined.reserve(sets.size());
@@ -1151,7 +1181,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // the wave's launches are ranked by FLOPs into launch priorities, so the
   // largest gets the SMs first and smaller ones fill the SMs it frees in its
   // tail.
-  const bool soft_groups = fused && !s->auto_plan && s->groups.size() > 1;
+  const bool soft_groups = fused && !join_launches && s->groups.size() > 1;
   if (fused) {
     for (size_t t0 = 0; t0 < sets.size();) {
       size_t t1 = t0;
@@ -1291,7 +1321,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // complete, so those runs keep the streams.
   int n_launches = 0;
   for (const LaunchSet& ls : sets) n_launches += ls.degenerate ? 0 : 1;
-  const bool one_stream = fused && (t_early || s->auto_plan) && n_launches >= 2;
+  const bool one_stream = fused && (t_early || join_launches) && n_launches >= 2;
   // A run of the dynamic logic without inputs_ready also goes out on
   // streams[0] alone: its first launch waits for the work queued before the
   // run, and lets the next launch start only after that (late_trigger), so the
@@ -1300,7 +1330,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // or B.  Their epilogues still wait for the launch before.  (Not in a traced
   // run, whose stamps are then those of one launch at a time, nor under a
   // caller's own wait limit, which would come to cover the launch before.)
-  const bool chain = one_stream && !t_early && s->auto_plan && t_pdl && !t_trace && t_wait_ns == 0;
+  const bool chain = one_stream && !t_early && join_launches && t_pdl && !t_trace && t_wait_ns == 0;
   bool chained = false;
   if (one_stream) lead = sets.size();
   std::vector<size_t> order;
@@ -1374,7 +1404,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
         chained = true;
       }
       // launches that follow one another on one stream each take the whole GPU
-      const bool whole = s->auto_plan && one_stream;
+      const bool whole = join_launches && one_stream;
       if (ls.n == 1 && !ls.mixed) {
         const int i = ls.members[0];
         st = launch_gemm(*d, s->gemms[i], A[i], B[i], C[i], ws, stream, whole ? 1e6 : ls.scale);

@@ -106,3 +106,28 @@ def test_mixed_launch_has_two_ctas_per_sm(cuda_ok, wide, out):
     assert kinds == [kind, 8]
     one = wide and out == F32
     assert _all_at_once(plan, shapes, out, sms if one else 2 * sms, inputs_ready=True)
+
+
+@pytest.mark.parametrize("out", [F32, BF16])
+@pytest.mark.parametrize("ready", [False, True])
+def test_cluster_reduced_launches_stay_apart(cuda_ok, ready, out):
+    """Two launches of which K splits that clusters reduce are two thirds stay two; with less they join."""
+    # (M, N, K, kind, split): 48 of 59 units split 4; 32 of 43; two splits of one kind; 16 of 43; split 2
+    for specs, want in (([(122, 1536, 2624, 2, 4), (38, 704, 256, 0, 1)], [48, 11]),
+                        ([(122, 1024, 2624, 2, 4), (38, 704, 256, 0, 1)], [32, 11]),
+                        ([(60, 1024, 1472, 8, 8), (41, 512, 1600, 8, 4)], [64, 16]),
+                        ([(122, 512, 2624, 2, 4), (38, 1728, 256, 0, 1)], [43]),
+                        ([(122, 1536, 2624, 2, 2), (38, 704, 256, 0, 1)], [35])):
+        shapes = [s[:3] for s in specs]
+        entries, descs = [], []
+        for M, N, K, kind, split in specs:
+            d = G.desc(M, N, K, out)
+            key = G.goldy_bucket_key(d)
+            entries.append((((key >> 24) & 255, (key >> 16) & 255, (key >> 8) & 255, key & 255), 2,
+                            [G.variant_id(kind, split, 1)] * 5))
+            descs.append(d)
+        lut = G.goldy_lut_from_memory(P.write_lut(entries, G.goldy_variant_count(), 152))
+        plan = G.goldy_plan(descs, lut, G.GOLDY_PLAN_AUTO | G.GOLDY_PLAN_FUSED)
+        got = [G.goldy_variant_info_get(G.goldy_schedule_entry(plan, i)[1]) for i in range(2)]
+        assert [(v["kind"], v["split_k"]) for v in got] == [s[3:] for s in specs]
+        assert sorted(_run(plan, shapes, out, inputs_ready=ready), reverse=True) == sorted(want, reverse=True)
