@@ -177,6 +177,7 @@ namespace goldy {
 struct DealtUnits {
   std::vector<int> members;
   int bins = 0;
+  bool round_robin = false;   // no shares: round-robin is as good
   std::vector<uint16_t> rounds, first;
 };
 constexpr size_t kMaxDealt = 16;   // launches kept per plan (two per run, for each grid size seen)

@@ -131,3 +131,51 @@ def test_cluster_reduced_launches_stay_apart(cuda_ok, ready, out):
         got = [G.goldy_variant_info_get(G.goldy_schedule_entry(plan, i)[1]) for i in range(2)]
         assert [(v["kind"], v["split_k"]) for v in got] == [s[3:] for s in specs]
         assert sorted(_run(plan, shapes, out, inputs_ready=ready), reverse=True) == sorted(want, reverse=True)
+
+
+def _table_plan(specs, out):
+    """Fused AUTO plan of (M, N, K, kind, split), each its own table entry, all at once."""
+    entries, descs = {}, []
+    for M, N, K, kind, split in specs:
+        d = G.desc(M, N, K, out)
+        key = G.goldy_bucket_key(d)
+        key = ((key >> 24) & 255, (key >> 16) & 255, (key >> 8) & 255, key & 255)
+        entries[key] = (key, 8, [G.variant_id(kind, split, 1)] * 5)
+        descs.append(d)
+    lut = G.goldy_lut_from_memory(P.write_lut(entries.values(), G.goldy_variant_count(), 152))
+    plan = G.goldy_plan(descs, lut, G.GOLDY_PLAN_AUTO | G.GOLDY_PLAN_FUSED)
+    got = [G.goldy_variant_info_get(G.goldy_schedule_entry(plan, i)[1]) for i in range(len(specs))]
+    assert [(v["kind"], v["split_k"]) for v in got] == [s[3:] for s in specs]
+    return plan
+
+
+def _units(specs, out, **opts):
+    """Units of every CTA, launch by launch, of one traced run; its results are checked."""
+    plan = _table_plan(specs, out)
+    A = [wl.integer_matrix(s[0], s[2], 8200 + i) for i, s in enumerate(specs)]
+    B = [wl.integer_matrix(s[2], s[1], 8220 + i) for i, s in enumerate(specs)]
+    launch = Launch(plan, A, B, [out] * len(specs))
+    trace = torch.zeros(1024 * 16, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    G.goldy_run_ex(plan, *launch.ptrs(), launch.ws.data_ptr(), launch.ws_bytes,
+                   [s.cuda_stream for s in launch.streams], trace=trace.data_ptr(), trace_ctas=1024, **opts)
+    for a, b, c in zip(A, B, launch.results()):
+        want = torch.matmul(a.cuda().double(), b.cuda().double()).to(c.dtype).cpu()
+        assert torch.equal(c, want)
+    rows = trace.view(1024, 16).cpu()
+    counts, at = [], 0
+    while at < 1024 and int(rows[at, 0]) != 0:
+        grid = int(rows[at, 12])
+        counts.append(rows[at:at + grid, 14].tolist())
+        at += grid
+    return counts
+
+
+def test_short_units_of_a_last_round_are_spread(cuda_ok):
+    """150 pair tiles of 34 K blocks, 6 of 15 and 2 of 4 on 76 pairs: round-robin, at most three to a pair."""
+    specs = [(1289, 6208, 2176, 10, 1), (150, 1472, 960, 10, 1), (216, 448, 256, 10, 1), (66, 1280, 2240, 0, 1)]
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the numbers are those of 152 SMs")
+    pair, single = sorted(_units(specs, F32, inputs_ready=True), key=len, reverse=True)
+    assert len(pair) == 152 and sum(pair) == 2 * 158 and max(pair) == 3 and min(pair) == 2
+    assert len(single) == 20
