@@ -180,6 +180,11 @@ struct DealtUnits {
   bool round_robin = false;   // no shares: round-robin is as good
   std::vector<uint16_t> rounds, first;
 };
+// The pairs that the pair launch of a joined run leaves to itself (see
+// pair_limit in runtime.cu), for an SM count.
+struct PairLimit {
+  int sms = 0, pairs = 0;
+};
 constexpr size_t kMaxDealt = 16;   // launches kept per plan (two per run, for each grid size seen)
 }  // namespace goldy
 
@@ -194,6 +199,7 @@ struct goldy_schedule {
   goldy::Runtime* rt = nullptr;   // created on first goldy_run
   mutable std::mutex dealt_mu;    // guards dealt
   mutable std::vector<goldy::DealtUnits> dealt;
+  mutable std::vector<goldy::PairLimit> pair_limits;   // at most kMaxDealt, under dealt_mu too
 };
 
 // A GEMM co-scheduled with an element-wise add (planner.cpp builds it,

@@ -686,9 +686,10 @@ int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, i
 }
 
 // scale > 0: the launch's grid cap is its variant's cap times `scale` (set for
-// heterogeneous fused waves, see goldy_run_ex), at most the whole GPU.
+// heterogeneous fused waves, see goldy_run_ex), at most the whole GPU.  limit >
+// 0: at most so many CTAs.
 goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, const void* B, void* C, uint8_t* ws,
-                         cudaStream_t stream, double scale = 0.0) {
+                         cudaStream_t stream, double scale = 0.0, int limit = 0) {
   if (degenerate(gp)) return launch_degenerate(gp, C, stream);
   const int out_bf16 = gp.desc.c_dtype == GOLDY_BF16 ? 1 : 0;
   const int planned = shape_kind(gp);
@@ -697,6 +698,7 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
   if (st != GOLDY_OK) return st;
   int64_t cap = std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(gp.variant).rc_div);
   if (scale > 0.0) cap = std::min<int64_t>(int64_t(ctas) * sms(d), std::max<int64_t>(1, int64_t(double(cap) * scale)));
+  if (limit > 0) cap = std::min<int64_t>(cap, limit);
   const int kind = run_kind(d, planned, out_bf16, 0, gp.units, gp.split, cap);
   if (kind != planned && cap >= sms(d)) cap = 2 * int64_t(sms(d));
   const KindInfo& k = kKinds[kind];
@@ -819,6 +821,56 @@ void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* m
   if (s->dealt.size() < kMaxDealt) s->dealt.push_back(std::move(d));
 }
 
+// Pairs for the pair launch of a joined run whose other launches have `others`
+// CTAs: the SMs that those leave free, if the launch ends as early with them
+// (by unit_cost, within 4%) as with all SMs; 0: all of them.  The other launches
+// then run beside it instead of behind it, and the next run's CTAs find SMs free
+// (77 pair tiles, two rounds on 76 pairs and on 58, next to 36 CTAs with K split
+// 4: 16.4 -> 13.3 us with inputs_ready; 80 next to 54: 20.9 -> 16.2; 100 next
+// to 27: 16.1 -> 12.3).  With fewer units to a
+// round the same bound would add a round to the longest launch (104 pair tiles
+// next to 36 CTAs, w/o inputs_ready: 49 -> 64 us).
+int pair_limit(const goldy_schedule* s, const int* members_in, int count, int64_t others, int sm_count) {
+  {
+    std::lock_guard<std::mutex> lock(s->dealt_mu);
+    for (const PairLimit& l : s->pair_limits)
+      if (l.sms == sm_count) return l.pairs;
+  }
+  int members[kMaxFused];
+  std::copy_n(members_in, count, members);
+  std::stable_sort(members, members + count,
+                   [&](int a, int b) { return unit_cost(s->gemms[a]) > unit_cost(s->gemms[b]); });
+  int64_t units[kMaxFused], total = 0;
+  double cost[kMaxFused];
+  bool rotate[kMaxFused];
+  for (int j = 0; j < count; ++j) {
+    units[j] = s->gemms[members[j]].units;
+    cost[j] = unit_cost(s->gemms[members[j]]);
+    rotate[j] = false;
+    total += units[j];
+  }
+  const int all = std::min(sm_count / 2, kMaxBins), left = int(std::max<int64_t>(0, sm_count - others)) / 2;
+  auto longest = [&](int bins) {
+    int32_t rounds[kMaxFused], first[kMaxFused * (kMaxBins + 1)];
+    assign_units(count, units, cost, rotate, bins, rounds, first);
+    double most = 0.0;
+    for (int b = 0; b < bins; ++b) {
+      double sum = 0.0;
+      for (int j = 0; j < count; ++j)
+        sum += cost[j] * double(first[j * (bins + 1) + b + 1] - first[j * (bins + 1) + b]);
+      most = std::max(most, sum);
+    }
+    return most;
+  };
+  PairLimit l;
+  l.sms = sm_count;
+  if (left > 0 && left < all && total > left && total <= int64_t(1) << 20 && longest(left) <= 1.04 * longest(all))
+    l.pairs = left;
+  std::lock_guard<std::mutex> lock(s->dealt_mu);
+  if (s->pair_limits.size() < kMaxDealt) s->pair_limits.push_back(l);
+  return l.pairs;
+}
+
 // CTAs per SM of a launch that mixes tile shapes: two when its units outnumber
 // the SMs (with fewer, a second CTA per SM only halves each unit's ring: 106
 // units 9.7 -> 11.3 us) and it runs with inputs_ready or behind another launch
@@ -848,10 +900,10 @@ int set_ctas(const DeviceState& d, const goldy_schedule* s, const int* members, 
 // that reads the tile shape per GEMM.  The grid cap is the sum of the members'
 // own caps (each GO-Kernel keeps the share of the GPU it was tuned for), at
 // most the whole GPU; `whole`: the whole GPU (a launch that carries several
-// waves of a run, or several kinds).
+// waves of a run, or several kinds); limit > 0: at most so many CTAs.
 goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* members_in, int count, bool mixed,
                           bool whole, const void* const* A, const void* const* B, void* const* C, uint8_t* ws,
-                          cudaStream_t stream, double scale = 0.0) {
+                          cudaStream_t stream, double scale = 0.0, int limit = 0) {
   const GemmPlan& g0 = s->gemms[members_in[0]];
   const int out_bf16 = g0.desc.c_dtype == GOLDY_BF16 ? 1 : 0;
   int64_t units = 0;
@@ -880,6 +932,7 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
     cap += std::max<int64_t>(1, int64_t(ctas) * sms(d) / variant_of(s->gemms[members_in[j]].variant).rc_div);
   if (scale > 0.0) cap = std::max<int64_t>(1, int64_t(double(cap) * scale));
   cap = whole ? int64_t(ctas) * sms(d) : std::min<int64_t>(cap, int64_t(ctas) * sms(d));
+  if (limit > 0) cap = std::min<int64_t>(cap, limit);
   const int kind = mixed ? planned : run_kind(d, planned, out_bf16, 1, units, split, cap);
   if (kind != planned && cap >= sms(d)) cap = 2 * int64_t(sms(d));
   const KindInfo& k = kKinds[kind];
@@ -1352,6 +1405,23 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // caller's own wait limit, which would come to cover the launch before.)
   const bool chain = one_stream && !t_early && join_launches && t_pdl && !t_trace && t_wait_ns == 0;
   bool chained = false;
+  int limit = 0;                             // CTAs of the pair launch (see pair_limit)
+  if (join_launches && one_stream) {
+    int64_t others = 0;
+    const LaunchSet* pair = nullptr;
+    bool one_pair = true;
+    for (const LaunchSet& ls : sets) {
+      if (ls.degenerate) continue;
+      const bool is_pair = kKinds[s->gemms[ls.members[0]].kind].pair != 0;
+      if (is_pair) {
+        one_pair = !pair;
+        pair = &ls;
+      }
+      for (int j = 0; j < ls.n && !is_pair; ++j) others += s->gemms[ls.members[j]].units;
+    }
+    if (pair && one_pair && others > 0 && others < sms(*d))
+      limit = 2 * pair_limit(s, pair->members, pair->n, others, sms(*d));
+  }
   if (one_stream) lead = sets.size();
   std::vector<size_t> order;
   order.reserve(sets.size());
@@ -1427,9 +1497,11 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       const bool whole = join_launches && one_stream;
       if (ls.n == 1 && !ls.mixed) {
         const int i = ls.members[0];
-        st = launch_gemm(*d, s->gemms[i], A[i], B[i], C[i], ws, stream, whole ? 1e6 : ls.scale);
+        st = launch_gemm(*d, s->gemms[i], A[i], B[i], C[i], ws, stream, whole ? 1e6 : ls.scale,
+                         kKinds[s->gemms[i].kind].pair ? limit : 0);
       } else {
-        st = launch_fused(*d, s, ls.members, ls.n, ls.mixed, ls.whole || whole, A, B, C, ws, stream, ls.scale);
+        st = launch_fused(*d, s, ls.members, ls.n, ls.mixed, ls.whole || whole, A, B, C, ws, stream, ls.scale,
+                          kKinds[s->gemms[ls.members[0]].kind].pair ? limit : 0);
       }
       t_prio = kNoPriority;
       t_started = nullptr;

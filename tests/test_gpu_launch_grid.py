@@ -179,3 +179,16 @@ def test_short_units_of_a_last_round_are_spread(cuda_ok):
     pair, single = sorted(_units(specs, F32, inputs_ready=True), key=len, reverse=True)
     assert len(pair) == 152 and sum(pair) == 2 * 158 and max(pair) == 3 and min(pair) == 2
     assert len(single) == 20
+
+
+@pytest.mark.parametrize("ready", [False, True])
+def test_pair_launch_leaves_room_beside_it(cuda_ok, ready):
+    """77 pair tiles take two rounds on 76 pairs and on 58: next to 36 CTAs they take 58.  With one tile more
+    than two rounds of 58, or with one tile to a pair of 76, they take all."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the numbers are those of 152 SMs")
+    small = (79, 384, 2816, 6, 4)            # 36 units
+    for tiles_n, tiles_m, want in ((11, 7, 2 * 58), (29, 4, 2 * 58), (39, 3, 2 * 76), (25, 3, 2 * 75)):
+        specs = [(256 * tiles_m - 6, 256 * tiles_n - 64, 896, 10, 1), small]
+        grids = sorted((len(u) for u in _units(specs, F32, inputs_ready=ready)), reverse=True)
+        assert grids == [want, 36], (tiles_n, tiles_m)
