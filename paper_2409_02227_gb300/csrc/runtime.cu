@@ -1198,6 +1198,28 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       apart = by_split.size() == 2;
       if (apart) sets.swap(by_split);
     }
+    // In a prepared run without inputs_ready, two launches on two streams also
+    // stay apart where they run side by side: all units fit on the GPU at once,
+    // or the pair launch needs no more rounds on the SMs that the other leaves.
+    // Joined, each replay waits for the second stream before it starts (see
+    // `ordered` below), which costs more than the second launch: 47 units in two
+    // launches 12.7 -> 10.3 us, 118 12.2 -> 10.3, 77 pair tiles and 36 units 22.5
+    // -> 20.5.  (A goldy_run is enqueued no faster than it runs, so that wait is
+    // over by then: 79 units joined 8.7 us, apart 11.4.)
+    if (!apart && t_rec && !t_early && sets.size() == 2 && (sets[0].slot | sets[1].slot) != 0 && !sets[0].degenerate &&
+        !sets[1].degenerate) {
+      int64_t units_of[2] = {0, 0}, sms_of[2];
+      bool pair[2];
+      for (int t = 0; t < 2; ++t) {
+        pair[t] = kKinds[s->gemms[sets[t].members[0]].kind].pair != 0;
+        for (int j = 0; j < sets[t].n; ++j) units_of[t] += s->gemms[sets[t].members[j]].units;
+        sms_of[t] = units_of[t] * (pair[t] ? 2 : 1);
+      }
+      apart = sms_of[0] + sms_of[1] <= sms(*d);
+      for (int t = 0; t < 2 && !apart; ++t)
+        apart = pair[t] && !pair[1 - t] && units_of[1 - t] < sms(*d) &&
+                pair_limit(s, sets[t].members, sets[t].n, units_of[1 - t], sms(*d)) > 0;
+    }
   }
   const bool join_launches = fused && s->auto_plan && !apart && sets.size() > 1;
   if (join_launches) {
