@@ -741,8 +741,11 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
 // such units: per K block a 256-wide pair tile takes 270 ns of tensor core
 // time (half that for 128 columns), a single CTA's operands arrive at about 85
 // bytes/ns, a tile leaves at about 45 bytes/ns (each SM's share of the memory
-// rate).  Only the ratios matter.
-double unit_cost(const GemmPlan& gp) {
+// rate).  `dealt`: for shares of one CTA per SM, where a single CTA's loads and
+// stores half overlap (a 128 x 256 fp32 tile of 5 K blocks, 2.9 us each way,
+// takes 6.3 us: with the slower one alone the CTAs that got 14 of them ended at
+// 89 us, the others at 56 to 61).  Only the ratios matter.
+double unit_cost(const GemmPlan& gp, bool dealt = true) {
   const KindInfo& k = kKinds[shape_kind(gp)];
   const goldy_gemm_desc& g = gp.desc;
   const double rows = double(g.M) / double(gp.tiles_m), cols = double(g.N) / double(gp.tiles_n);
@@ -755,7 +758,8 @@ double unit_cost(const GemmPlan& gp) {
   } else {
     per_kb = std::max(270.0 * k.mma_n / 256.0, (rows + cols) * 128.0 / 85.0);
   }
-  return std::max(kb * per_kb, out) + 500.0;
+  const double load = kb * per_kb;
+  return std::max(load, out) + (dealt && !k.pair ? 0.5 * std::min(load, out) : 0.0) + 500.0;
 }
 
 // Equal shares of a launch's units for its `bins` CTAs (pairs); `members`
@@ -954,8 +958,10 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   int members[kMaxFused];
   for (int j = 0; j < count; ++j) members[j] = members_in[j];
   if (cluster == 0) {
-    std::stable_sort(members, members + count,
-                     [&](int a, int b) { return unit_cost(s->gemms[a]) > unit_cost(s->gemms[b]); });
+    const bool dealt = !(mixed && ctas == 2);
+    std::stable_sort(members, members + count, [&](int a, int b) {
+      return unit_cost(s->gemms[a], dealt) > unit_cost(s->gemms[b], dealt);
+    });
     deal_units(p.shares, s, members, count, int(pair ? grid / 2 : grid));
     if (mixed && ctas == 2) p.shares.on = 2;
   }
