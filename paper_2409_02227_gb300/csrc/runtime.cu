@@ -88,6 +88,7 @@ thread_local bool t_pdl = true;
 // (first launch of the run only).
 thread_local int32_t t_early = 0;
 thread_local bool t_named = false;  // an explicit schedule: its launches run the kinds it names
+thread_local bool t_alone = false;  // the run's only launch: no other of the run has SMs to share with it
 thread_local int32_t t_late = 0;    // LaunchParams::late_trigger of the next launch
 thread_local uint64_t t_wait_ns = 0;
 thread_local int32_t t_stall = 0;
@@ -664,10 +665,13 @@ unsigned long long* trace_for(unsigned grid) {
 // `cap` is the planned kind's grid cap.  A launch that may not use the whole GPU
 // keeps its share: it takes the two-per-SM kind only where the cap does not bind
 // (so that its grid is the same, of CTAs half the size), never to run a second
-// round's units on more SMs than it was given.
+// round's units on more SMs than it was given.  Several GEMMs in a run's only
+// launch have nothing beside them: there twice the cap of half-size CTAs is the
+// same share (three 216 x 576 x 1664 split 4 at a quarter of the GPU each, with
+// inputs_ready: 240 units on 114 CTAs 11.8 us, on 228 half-size ones 9.6).
 int run_kind(DeviceState& d, int kind, int out_bf16, int fused, int64_t units, int split, int64_t cap) {
-  const bool whole = cap >= sms(d);
-  if (t_named || (!t_early && (!whole || units <= sms(d))) || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 ||
+  const bool whole = t_alone || cap >= sms(d);
+  if (t_named || (!t_early && (!whole || units <= cap || units > 2 * cap)) || kKinds[kind].pair || kKinds[kind].ctas_per_sm != 1 ||
       kKinds[kind].mma_n > 128)
     return kind;
   const int twin = kind + 1;
@@ -700,7 +704,7 @@ goldy_status launch_gemm(DeviceState& d, const GemmPlan& gp, const void* A, cons
   if (scale > 0.0) cap = std::min<int64_t>(int64_t(ctas) * sms(d), std::max<int64_t>(1, int64_t(double(cap) * scale)));
   if (limit > 0) cap = std::min<int64_t>(cap, limit);
   const int kind = run_kind(d, planned, out_bf16, 0, gp.units, gp.split, cap);
-  if (kind != planned && cap >= sms(d)) cap = 2 * int64_t(sms(d));
+  if (kind != planned && (t_alone || cap >= sms(d))) cap *= 2;
   const KindInfo& k = kKinds[kind];
   if (gp.units > int64_t(1) << 30) return fail(GOLDY_ERR_UNSUPPORTED, "too many tiles in one GEMM");
 
@@ -938,7 +942,7 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   cap = whole ? int64_t(ctas) * sms(d) : std::min<int64_t>(cap, int64_t(ctas) * sms(d));
   if (limit > 0) cap = std::min<int64_t>(cap, limit);
   const int kind = mixed ? planned : run_kind(d, planned, out_bf16, 1, units, split, cap);
-  if (kind != planned && cap >= sms(d)) cap = 2 * int64_t(sms(d));
+  if (kind != planned && (t_alone || cap >= sms(d))) cap *= 2;
   const KindInfo& k = kKinds[kind];
   const void* fn = mixed ? kernel_fn_set(out_bf16, ctas) : kernel_fn(kind, out_bf16, 1);
   static thread_local LaunchParams<kMaxFused> p;   // ~12 KB: keep it off the stack
@@ -1042,6 +1046,7 @@ struct RunOptionsReset {
     t_pdl = true;
     t_early = 0;
     t_named = false;
+    t_alone = false;
     t_late = 0;
     t_wait_ns = 0;
     t_stall = 0;
@@ -1423,6 +1428,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   int n_launches = 0;
   for (const LaunchSet& ls : sets) n_launches += ls.degenerate ? 0 : 1;
   const bool one_stream = fused && (t_early || join_launches) && n_launches >= 2;
+  t_alone = fused && n_launches == 1 && s->gemms.size() > 1;
   // A run of the dynamic logic without inputs_ready also goes out on
   // streams[0] alone: its first launch waits for the work queued before the
   // run, and lets the next launch start only after that (late_trigger), so the

@@ -54,11 +54,14 @@ def test_planned_launch_keeps_its_share(cuda_ok, kind, tile_cols, rc, ready):
 @pytest.mark.parametrize("ready", [False, True])
 def test_fused_launch_keeps_the_sum_of_its_shares(cuda_ok, ready):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    for rc, tiles in ((4, sms // 2), (4, sms // 4 - 2), (2, sms // 2 + 10)):
+    for rc, tiles in ((4, sms // 4 - 2), (4, sms // 4), (4, sms // 4 + 1), (4, sms // 2), (4, sms // 2 + 1),
+                      (2, sms // 2 + 10), (2, sms), (2, sms + 1)):
         cap = 2 * (sms // rc)
         shapes = [(100, tiles * 128, 136), (100, tiles * 128, 136)]
         units = 2 * tiles
-        want = units if cap >= sms and units <= 2 * sms else min(units, cap)
+        # the run's only launch: twice as many half-size CTAs are the same share
+        half = units <= 2 * sms if ready else cap < units <= 2 * cap
+        want = min(units, 2 * cap if half else cap)
         assert _run(_plan(shapes, [2, 2], rc, G.GOLDY_PLAN_FUSED), shapes, inputs_ready=ready) == [want]
 
 
