@@ -1191,7 +1191,10 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // split 4 9.8 -> 7.3; 58 x 960 x 384 next to 33 x 320 x 640 split 8 (f32) 6.2 -> 4.5.
   // At least two thirds of the units, split 4 or more: with half of them split
   // (22 x 896 x 320 next to 24 x 384 x 320 split 5) apart is slower, 5.5 -> 7.2,
-  // and a split of 2 (38 of 47 units) exchanges too little, 4.8 -> 5.2.
+  // and a split of 2 (38 of 47 units) exchanges too little, 4.8 -> 5.2.  (One
+  // launch of several splits is only divided with inputs_ready: on two streams
+  // the fork and join cost as much, 36 units split 4 next to 3 unsplit ones 15.6
+  // -> 16.3.)
   uint32_t slots = 0;                        // the slots on whose streams these launches would go out
   for (const LaunchSet& ls : sets) slots |= 1u << ls.slot;
   bool apart = false;
@@ -1203,7 +1206,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       units += gp.units;
       if (gp.split >= 4) reducible += gp.units;
     }
-    if (single && units <= sms(*d) && 3 * reducible >= 2 * units) {
+    if (single && (t_early || sets.size() == 2) && units <= sms(*d) && 3 * reducible >= 2 * units) {
       std::vector<LaunchSet> by_split;
       make_sets(by_split, true);
       apart = by_split.size() == 2;
