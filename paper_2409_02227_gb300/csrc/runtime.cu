@@ -1308,8 +1308,9 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       // Plans of several groups keep the full c/m: there the same bound
       // measured 5-28% slower (the over-subscribed first group's CTAs take
       // SMs as they free up, ahead of the later groups' launches).
+      // (A joined run's launches each have the whole GPU: no scale.)
       double fit = 1e30;
-      if (kernels > 1 && !soft_groups) {
+      if (kernels > 1 && !soft_groups && !join_launches) {
         struct Need {
           double units, cap, ctas;   // CTAs of work, the launch's own cap, CTAs per SM
         };
