@@ -885,7 +885,7 @@ int pair_limit(const goldy_schedule* s, const int* members_in, int count, int64_
 // of its run, where the CTAs of consecutive launches overlap (nine GEMMs, 426
 // units: 28.3 -> 19.3 us; 257 units 16.8 -> 9.6; a second launch of 302 units,
 // its run 69.4 -> 57.9).  The kernel for two keeps no staging buffers, so C's
-// rows have to be aligned.  One, too, where 256-column tiles write f32: there
+// rows (and its batch entries) have to be aligned.  One, too, where 256-column tiles write f32: there
 // is room for one accumulator that wide, so each tile's MMAs wait for the
 // 128 KB that the tile before stores from registers (sets of 8 to 14 GEMMs with
 // f32 C and 225 to 1428 units: two per SM 22.8, 34.8, 76, 92, 110, 134 us, one
@@ -898,7 +898,9 @@ int set_ctas(const DeviceState& d, const goldy_schedule* s, const int* members, 
     const GemmPlan& gp = s->gemms[members[j]];
     const size_t es = gp.desc.c_dtype == GOLDY_BF16 ? 2 : 4;
     if (es == 4 && stage_bytes(kKinds[shape_kind(gp)]) > stage_bytes(kKinds[2])) return 1;
-    if (!kKinds[shape_kind(gp)].swap_ab && (!aligned(C[members[j]], 16) || size_t(gp.desc.ldc) * es % 16 != 0)) return 1;
+    const bool rows = aligned(C[members[j]], 16) && size_t(gp.desc.ldc) * es % 16 == 0 &&
+                      (gp.desc.batch <= 1 || size_t(gp.desc.stride_c) * es % 16 == 0);
+    if (!rows && !kKinds[shape_kind(gp)].swap_ab) return 1;
   }
   return 2;
 }

@@ -195,3 +195,38 @@ def test_pair_launch_leaves_room_beside_it(cuda_ok, ready):
         specs = [(256 * tiles_m - 6, 256 * tiles_n - 64, 896, 10, 1), small]
         grids = sorted((len(u) for u in _units(specs, F32, inputs_ready=ready)), reverse=True)
         assert grids == [want, 36], (tiles_n, tiles_m)
+
+
+@pytest.mark.parametrize("stride,per_sm", [(200 * 1024, 2), (200 * 1024 + 1, 1)])
+def test_mixed_launch_with_unaligned_batch_entries(cuda_ok, stride, per_sm):
+    """Two CTAs per SM want C's rows 16-byte aligned in every entry of a strided batch."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    M, N, K, batch = 200, 1024, 136, 12       # 192 units of 128 x 128
+    descs = [G.desc(M, N, K, F32, batch=batch, stride_c=stride), G.desc(60, 2048, 200, F32)]
+    entries = []
+    for d, kind in zip(descs, (2, 8)):
+        key = G.goldy_bucket_key(d)
+        entries.append((((key >> 24) & 255, (key >> 16) & 255, (key >> 8) & 255, key & 255), 2,
+                        [G.variant_id(kind, 1, 1)] * 5))
+    lut = G.goldy_lut_from_memory(P.write_lut(entries, G.goldy_variant_count(), 152))
+    plan = G.goldy_plan(descs, lut, G.GOLDY_PLAN_AUTO | G.GOLDY_PLAN_FUSED)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    new = lambda *s: torch.randint(-3, 4, s, generator=gen, device="cuda").bfloat16()
+    A, B = [new(batch, M, K), new(60, 200)], [new(batch, K, N), new(200, 2048)]
+    C0 = torch.full((batch * stride,), -7.0, device="cuda")
+    C = [torch.as_strided(C0, (batch, M, N), (stride, N, 1)), torch.empty((60, 2048), device="cuda")]
+    _, _, n_streams, ws_bytes = G.goldy_schedule_query(plan)
+    ws = torch.zeros(max(ws_bytes, 256), dtype=torch.uint8, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(n_streams)]
+    trace = torch.zeros(1024 * 16, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    G.goldy_run_ex(plan, [a.data_ptr() for a in A], [b.data_ptr() for b in B], [c.data_ptr() for c in C],
+                   ws.data_ptr(), ws_bytes, [s.cuda_stream for s in streams], trace=trace.data_ptr(), trace_ctas=1024,
+                   inputs_ready=True)
+    torch.cuda.synchronize()
+    assert G.goldy_device_error(clear=True) == 0
+    for a, b, c in zip(A, B, C):
+        assert torch.equal(c.double(), a.double() @ b.double())
+    for e in range(batch - 1):                # nothing written between the entries
+        assert bool((C0[e * stride + M * N:(e + 1) * stride] == -7.0).all())
+    assert int(trace[12]) == min(192 + 16, per_sm * sms)
