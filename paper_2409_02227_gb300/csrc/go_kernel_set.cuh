@@ -17,9 +17,10 @@
 // CTAS = 1, one CTA per SM: tensor memory holds two accumulators of 256 columns
 // whatever the tile's width; the operand ring is cut into stages of the
 // launch's widest tile (192 KB: 4 stages of 48 KB up to 8 of 24 KB or less).
-// CTAS = 2, two per SM, for runs with inputs_ready: half the ring and half the
-// tensor memory (two accumulators of 128 columns, or one of 256 when the launch
-// has tiles that wide), no staging buffers (tiles other than a CTA's last are
+// CTAS = 2, two per SM, for runs with inputs_ready and launches behind the first
+// of a run: half the ring and half the tensor memory (two accumulators of 128
+// columns, or one of 256 when a bf16 launch has tiles that wide; an fp32 launch
+// with such tiles runs one CTA per SM), no staging buffers (tiles other than a CTA's last are
 // stored from registers), so that the next run's CTAs load and multiply while
 // this run's finish.  The units, sorted longest first, go to the CTAs back and
 // forth (0 .. n-1, n-1 .. 0, ...), which balances the few units a CTA gets.
@@ -289,9 +290,10 @@ __global__ void __launch_bounds__(192, CTAS) go_gemm_set_kernel(const __grid_con
       // transposed), and whether any of this warp's accumulator rows do
       const int ncols = swap ? min(w.mma_n, w.m - m0) : min(w.mma_n, w.n - n0);
       const bool live = swap ? n0 + 32 * q < w.n : m0 + 32 * q < w.m;
-      // see go_gemm_kernel; the half ring holds 128 rows of 192 fp32 columns
-      const bool wide = !swap && w.split == 1 && walk.last() &&
-                        (CTAS == 1 || ncols * 128 * (OUT_BF16 ? 2 : 4) <= RING_BYTES);
+      // see go_gemm_kernel; a launch of two CTAs per SM has fp32 tiles of at most
+      // 128 columns (the host sees to it), which its half ring holds
+      static_assert(128 * (OUT_BF16 ? 256 * 2 : CTAS == 1 ? 256 * 4 : 128 * 4) <= RING_BYTES, "the ring holds a tile");
+      const bool wide = !swap && w.split == 1 && walk.last();
       if (wide) {
         stage_tile_wide<OUT_BF16>(cv, tiles_base, taddr, et, q, m0, ncols);
         wait_prev();

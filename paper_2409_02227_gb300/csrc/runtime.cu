@@ -991,6 +991,8 @@ goldy_status launch_fused(DeviceState& d, const goldy_schedule* s, const int* me
   p.stage_bytes = stage;
   p.stages = mixed ? std::min(kSetMaxStages, set_ring_bytes(ctas) / stage) : 0;
   p.acc_stages = stage > stage_bytes(kKinds[2]) ? 1 : 2;   // one 256-column accumulator, or two of 128
+  if (mixed && ctas == 2 && !out_bf16 && p.acc_stages == 1)
+    return fail(GOLDY_ERR_UNSUPPORTED, "256-column fp32 tiles need one CTA per SM");   // (see set_ctas)
   p.trace = trace_for(grid);
   cudaError_t e = launch_kernel(fn, grid, size_t(mixed ? set_smem_bytes(ctas) : smem_bytes(k)), stream, &p, sizeof(p),
                                 pair ? 2 : cluster);
