@@ -127,3 +127,75 @@ def test_joined_run_keeps_the_order_of_its_streams(cuda_ok, wave, how):
         for i, (M, N, K, _) in enumerate(specs):
             assert torch.equal(o[i].double(), a[i].double() @ B[i][:, :N].double()), (specs[i], how)
     del ex
+
+
+@pytest.mark.parametrize("how", ["run", "exec", "captured run"])
+def test_joined_run_reads_what_the_kernel_before_it_wrote(cuda_ok, how):
+    """The later launches of a joined run start while its first is still going on; their operands, written by
+    the kernel right before the run, have to be there all the same."""
+    specs = [(700, 2600, 1096, 10), (100, 1320, 4096, 2), (40, 1500, 2200, 8), (20, 600, 4000, 6)]
+    entries, descs = [], []
+    for M, N, K, kind in specs:
+        d = G.desc(M, N, K, F32, lda=K, ldb=(N + 7) // 8 * 8, ldc=N)
+        key = G.goldy_bucket_key(d)
+        entries.append((((key >> 24) & 255, (key >> 16) & 255, (key >> 8) & 255, key & 255), 4,
+                        [G.variant_id(kind, 1, 1)] * 5))
+        descs.append(d)
+    lut = G.goldy_lut_from_memory(P.write_lut(entries, G.goldy_variant_count(), 152))
+    plan = G.goldy_plan(descs, lut, G.GOLDY_PLAN_AUTO | G.GOLDY_PLAN_FUSED)
+    kinds = [G.goldy_variant_info_get(G.goldy_schedule_entry(plan, i)[1])["kind"] for i in range(len(specs))]
+    assert kinds == [s[3] for s in specs]    # one launch of the pair kernel, one of the others
+    _, _, n_streams, ws_bytes = G.goldy_schedule_query(plan)
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    new = lambda r, c: torch.randint(-3, 4, (r, c), generator=gen, device="cuda").bfloat16()
+    rounds = 8
+    # all A and all B in one buffer each round, so that one kernel writes them right before the run
+    sizes = [M * K + K * ((N + 7) // 8 * 8) for M, N, K, _ in specs]
+    src = [torch.cat([new(1, n)[0] for n in sizes]) for _ in range(rounds)]
+    buf = torch.zeros(sum(sizes), dtype=torch.bfloat16, device="cuda")
+
+    def views(t):
+        A, B, at = [], [], 0
+        for M, N, K, _ in specs:
+            ld = (N + 7) // 8 * 8
+            A.append(t[at:at + M * K].view(M, K))
+            B.append(t[at + M * K:at + M * K + K * ld].view(K, ld))
+            at += M * K + K * ld
+        return A, B
+
+    A, B = views(buf)
+    C = [torch.zeros((M, N), device="cuda") for M, N, K, _ in specs]
+    out = [[torch.zeros_like(c) for c in C] for _ in range(rounds)]
+    ws = torch.zeros(max(ws_bytes, 256), dtype=torch.uint8, device="cuda")
+    streams = [torch.cuda.Stream() for _ in range(n_streams)]
+    args = (plan, [a.data_ptr() for a in A], [b.data_ptr() for b in B], [c.data_ptr() for c in C], ws.data_ptr(),
+            ws_bytes, [s.cuda_stream for s in streams])
+    assert all(t.data_ptr() % 16 == 0 for t in A + B)
+    ex = G.goldy_exec_create(*args) if how == "exec" else None
+    launch = (lambda: G.goldy_exec_launch(ex)) if ex else (lambda: G.goldy_run(*args))
+    torch.cuda.synchronize()
+
+    def steps():
+        for r in range(rounds):
+            buf.copy_(src[r])
+            launch()
+            for c, o in zip(C, out[r]):
+                o.copy_(c)
+
+    if how == "captured run":
+        launch()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=streams[0]):
+            steps()
+        g.replay()
+    else:
+        with torch.cuda.stream(streams[0]):
+            steps()
+    torch.cuda.synchronize()
+    assert G.goldy_device_error(clear=True) == 0
+    for r in range(rounds):
+        a, b = views(src[r])
+        for i, (M, N, K, _) in enumerate(specs):
+            assert torch.equal(out[r][i].double(), a[i].double() @ b[i][:, :N].double()), (r, specs[i], how)
+    del ex
