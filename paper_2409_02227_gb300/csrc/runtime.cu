@@ -7,9 +7,9 @@
 // most CD GEMMs are in flight, each stream running its GEMMs back to back),
 // and joins back into streams[0] before the next group starts.  In the fused
 // launch mode the GEMMs of a wave that share a kernel kind go out as one
-// persistent launch over all their tiles instead, and a plan of the dynamic
-// logic as at most two launches (per output dtype) over the tiles of all its
-// GEMMs.  The whole run can be captured once into a CUDA graph and replayed
+// persistent launch over all their tiles instead, and most plans of the dynamic
+// logic as one launch per kernel family (CTA pair, single CTA), output dtype and
+// 16 GEMMs, over the tiles of all its GEMMs.  The whole run can be captured once into a CUDA graph and replayed
 // with one launch.
 //
 // Per GEMM the host encodes two TMA tensor maps (A and B), sizes the
@@ -808,18 +808,22 @@ void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* m
   d.members.assign(members, members + count);
   d.bins = bins;
   double dealt = 0.0, dealt_rr = 0.0;        // the longest bin's cost
-  for (int b = 0; b < bins; ++b) {
-    double share = 0.0, rr = 0.0;
-    int64_t at = 0;
-    for (int j = 0; j < count; ++j) {
-      const int32_t* f = first + int64_t(j) * (bins + 1) + b;
-      share += cost[j] * double(rounds[j] + f[1] - f[0]);
-      // units at .. at + units[j] - 1 of the launch; bin b has those = b modulo bins
-      rr += cost[j] * double((at + units[j] - b + bins - 1) / bins - (at - b + bins - 1) / bins);
-      at += units[j];
+  double share[kMaxBins] = {}, rr[kMaxBins] = {};
+  int at = 0;                                // the bin of GEMM j's first unit, round-robin
+  for (int j = 0; j < count; ++j) {
+    const int32_t* f = first + int64_t(j) * (bins + 1);
+    const int64_t whole = units[j] / bins;
+    const int rest = int(units[j] % bins);
+    for (int b = 0; b < bins; ++b) {
+      share[b] += cost[j] * double(rounds[j] + f[b + 1] - f[b]);
+      const int behind = b >= at ? b - at : b - at + bins;
+      rr[b] += cost[j] * double(whole + (behind < rest ? 1 : 0));
     }
-    dealt = std::max(dealt, share);
-    dealt_rr = std::max(dealt_rr, rr);
+    at = at + rest < bins ? at + rest : at + rest - bins;
+  }
+  for (int b = 0; b < bins; ++b) {
+    dealt = std::max(dealt, share[b]);
+    dealt_rr = std::max(dealt_rr, rr[b]);
   }
   d.round_robin = dealt_rr <= 1.04 * dealt && std::find(rotate, rotate + count, false) == rotate + count;
   d.rounds.assign(rounds, rounds + count);
@@ -837,7 +841,9 @@ void deal_units(UnitShares<kMaxFused>& sh, const goldy_schedule* s, const int* m
 // 4: 16.4 -> 13.3 us with inputs_ready; 80 next to 54: 20.9 -> 16.2; 100 next
 // to 27: 16.1 -> 12.3).  With fewer units to a
 // round the same bound would add a round to the longest launch (104 pair tiles
-// next to 36 CTAs, w/o inputs_ready: 49 -> 64 us).
+// next to 36 CTAs, w/o inputs_ready: 49 -> 64 us).  Not for a launch of over a
+// millisecond: the other's load and MMA roles start beside it and wait for its
+// end (by their epilogue) within the limit of every wait, two seconds.
 int pair_limit(const goldy_schedule* s, const int* members_in, int count, int64_t others, int sm_count) {
   {
     std::lock_guard<std::mutex> lock(s->dealt_mu);
@@ -872,8 +878,10 @@ int pair_limit(const goldy_schedule* s, const int* members_in, int count, int64_
   };
   PairLimit l;
   l.sms = sm_count;
-  if (left > 0 && left < all && total > left && total <= int64_t(1) << 20 && longest(left) <= 1.04 * longest(all))
-    l.pairs = left;
+  if (left > 0 && left < all && total > left && total <= int64_t(1) << 20) {
+    const double time = longest(left);
+    if (time <= 1e6 && time <= 1.04 * longest(all)) l.pairs = left;
+  }
   std::lock_guard<std::mutex> lock(s->dealt_mu);
   if (s->pair_limits.size() < kMaxDealt) s->pair_limits.push_back(l);
   return l.pairs;

@@ -230,3 +230,30 @@ def test_mixed_launch_with_unaligned_batch_entries(cuda_ok, stride, per_sm):
     for e in range(batch - 1):                # nothing written between the entries
         assert bool((C0[e * stride + M * N:(e + 1) * stride] == -7.0).all())
     assert int(trace[12]) == min(192 + 16, per_sm * sms)
+
+
+def test_long_pair_launch_takes_the_whole_gpu(cuda_ok):
+    """Next to 4 CTAs a pair launch ends within 4% on the SMs that they leave, but one of over a millisecond
+    does not leave them (the other launch would wait for it, loaded, for as long)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    small = (60, 512, 9216, 8, 1)             # 4 units
+    for M, want in ((4096, sms - 4), (20480, sms)):
+        specs = [(M, 8192, 8192, 10, 1), small]
+        plan = _table_plan(specs, BF16)
+        _, _, n_streams, ws_bytes = G.goldy_schedule_query(plan)
+        A = [torch.zeros((s[0], s[2]), dtype=torch.bfloat16, device="cuda") for s in specs]
+        B = [torch.zeros((s[2], s[1]), dtype=torch.bfloat16, device="cuda") for s in specs]
+        C = [torch.ones((s[0], s[1]), dtype=torch.bfloat16, device="cuda") for s in specs]
+        ws = torch.zeros(max(ws_bytes, 256), dtype=torch.uint8, device="cuda")
+        streams = [torch.cuda.Stream() for _ in range(n_streams)]
+        trace = torch.zeros(1024 * 16, dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        G.goldy_run_ex(plan, [t.data_ptr() for t in A], [t.data_ptr() for t in B], [t.data_ptr() for t in C],
+                       ws.data_ptr(), ws_bytes, [x.cuda_stream for x in streams], trace=trace.data_ptr(),
+                       trace_ctas=1024)
+        torch.cuda.synchronize()
+        assert G.goldy_device_error(clear=True) == 0
+        rows = trace.view(1024, 16).cpu()
+        rows = rows[rows[:, 0] != 0]
+        assert sorted(set(rows[:, 12].tolist())) == [4, want]
+        assert not any(bool(c.any()) for c in C)
