@@ -100,30 +100,29 @@ typedef struct goldy_graph goldy_graph;
 #define GOLDY_PLAN_DEFAULT 2
 #define GOLDY_PLAN_GO 3
 #define GOLDY_PLAN_FORCE_CD 4
-/* Launch-mode bit, combinable with any policy above.  FUSED with AUTO: a plan
- * whose waves (a group's members taken CD at a time) would need several
- * launches runs as one persistent launch of the CTA-pair kind's GEMMs and one
- * of all other kinds' (per output dtype, at most 16 GEMMs per launch), their
- * tiles dealt out to the GPU's CTAs in equal shares, longest first; both go
- * out on streams[0] alone, the largest first, each overlapping the previous
- * one's tail.  Without inputs_ready such a run starts after what was enqueued
- * before it on the streams that the waves' own launches would have used, and
- * what is enqueued there later starts after the run.  FUSED otherwise
- * (explicit schedules, the forced policies), and for a plan of a single
- * launch: within each group, the GEMMs of a wave that share a kernel kind and
- * output dtype go into ONE persistent launch over the concatenation of their
- * tiles (at most 16 GEMMs per launch); its grid cap is the sum of the members'
- * caps.  A wave's
- * launches carry launch priorities ranked by their FLOPs, and the first wave's
- * largest launch goes out first (outside a stream capture the other streams
- * also wait until all of its CTAs have begun).  Groups are not separated by a
- * join: the run forks once and joins once, and a later group's launches take
- * lower priorities, so they fill the SMs an earlier group frees.  Such a run
- * with goldy_run_opts.inputs_ready = 1 goes out on streams[0] alone instead,
- * each wave's largest launch first.  Without FUSED every GEMM is its own
- * launch on its slot's stream and the groups run one after another.  The plan
- * (groups, CDs, variants, slots) is the same, and so are the results, byte
- * for byte. */
+/* Launch-mode bit, combinable with any policy above.  FUSED: within each
+ * group, the GEMMs that run at the same time (a "wave" of CD members) and
+ * share a kernel kind and output dtype go into ONE persistent launch over the
+ * concatenation of their tiles (at most 16 GEMMs per launch); its grid cap is
+ * the sum of the members' caps.  A wave's launches carry launch priorities
+ * ranked by their FLOPs, and the first wave's largest launch goes out first
+ * (outside a stream capture the other streams also wait until all of its CTAs
+ * have begun).  Groups are not separated by a join: the run forks once and
+ * joins once, and a later group's launches take lower priorities, so they fill
+ * the SMs an earlier group frees.  Such a run with goldy_run_opts.inputs_ready
+ * = 1 goes out on streams[0] alone instead, each wave's largest launch first.
+ * FUSED with AUTO: a plan that would so need several launches runs as one
+ * persistent launch of the CTA-pair kind's GEMMs and one of all other kinds'
+ * (per output dtype, at most 16 GEMMs per launch), their tiles dealt out to
+ * the GPU's CTAs in equal shares, longest first; both go out on streams[0]
+ * alone, the largest first, each overlapping the previous one's tail.  Without
+ * inputs_ready such a run starts after what was enqueued before it on the
+ * streams that the separate launches would have used, and what is enqueued
+ * there later starts after the run.  Two launches that run side by side or
+ * whose K splits are reduced on chip may stay apart.  Without FUSED every GEMM
+ * is its own launch on its slot's stream and the groups run one after another.
+ * The plan (groups, CDs, variants, slots) is the same, and so are the results,
+ * byte for byte. */
 #define GOLDY_PLAN_FUSED 0x10
 
 #define GOLDY_MAX_GEMMS 64      /* GEMMs per plan */
@@ -288,8 +287,10 @@ void goldy_schedule_free(goldy_schedule* s);
  * max_streams.  Groups run in order (in GOLDY_PLAN_FUSED mode by launch
  * priority, see there); the run forks from streams[0] and joins back to it,
  * so work queued on streams[0] before the call happens before every GEMM and
- * work queued on streams[0] after it happens after all of them.  Slot k runs on streams[k].  Asynchronous: returns after launching;
- * no allocation, no synchronisation.  Errors: GOLDY_ERR_INVALID_ARG (null or
+ * work queued on streams[0] after it happens after all of them.  Slot k runs on
+ * streams[k] (in GOLDY_PLAN_FUSED mode see there; streams[0] is the one ordering
+ * point of every run).  Asynchronous: returns after launching; no allocation,
+ * no synchronisation.  Errors: GOLDY_ERR_INVALID_ARG (null or
  * misaligned pointers, too few streams, workspace too small),
  * GOLDY_ERR_CUDA (launch failure).  A kernel that gave up a bounded wait
  * shows up later through goldy_device_error(); the outputs of that run are
@@ -301,7 +302,7 @@ goldy_status goldy_run(const goldy_schedule* s, const void* const* A, const void
 
 /* Options of goldy_run_ex / goldy_graph_create_ex (all fields may be null).
  * ev_begin[i] / ev_end[i] (cudaEvent_t as void*, caller-created, one pair per
- * GEMM) are recorded on GEMM i's stream right before and right after its
+ * GEMM) are recorded on the stream of GEMM i's launch right before and right after its
  * kernel launch, so the caller can time each launch on the stream it runs on.
  * Inside a graph capture they become event-record nodes of the graph. */
 typedef struct goldy_run_opts {

@@ -14,10 +14,10 @@
 //     of the work, dealt out by the host longest units first.  The
 //     grid size is the variant's resource constraint: capping it is how a
 //     GO-Kernel leaves SMs to co-running GEMMs (Sec. 4.2.1).
-//   * warp 0 (one thread): TMA producer.  Per 64-wide K block it loads the
+//   * warp 0 (one elected thread issues): TMA producer.  Per 64-wide K block it loads the
 //     A tile (K-major, 128-byte swizzle) and the B tile (N-major, 128-byte
 //     swizzle) into a shared-memory ring of STAGES slots (mbarrier full/empty).
-//   * warp 1 (one thread): allocates tensor memory, issues tcgen05.mma
+//   * warp 1 (one elected thread issues): allocates tensor memory, issues tcgen05.mma
 //     (M = 128, N = MMA_N, K = 16 per instruction) into an fp32 accumulator
 //     in tensor memory, ACC accumulators deep so the epilogue of one tile
 //     overlaps the main loop of the next.
@@ -441,7 +441,7 @@ __device__ __forceinline__ void reduce_slice(const CView& w, const float4* tile_
 // than the barriers cost (bench set of 280 pair tiles: 50.0 -> 51.1 us).  Why
 // lanes along the columns: one row per lane wrote 4 bytes of each 32-byte
 // sector per instruction (777 x 1501 x 1003, fp32 rows 4-byte aligned: 19.2
-// -> 13.8 us).
+// -> 14.1 us).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kWarpChunk = 4096;    // 32 rows x 128 bytes: a warp's part of a chunk
 constexpr uint32_t kChunkBytes = 16384;  // 128 rows x 128 bytes

@@ -10,7 +10,7 @@
 // operands for 128 x 256 x 64 multiply-adds — two thirds of what the
 // single-CTA 128 x 256 tile needs — which keeps the tensor cores fed from L2.
 //
-// Roles per CTA (192 threads): warp 0 lane 0 loads (both CTAs; the odd CTA's
+// Roles per CTA (192 threads): warp 0 loads, one elected thread issuing (both CTAs; the odd CTA's
 // loads complete on the even CTA's barrier), warp 1 allocates tensor memory
 // jointly with the peer and, in the even CTA, issues the MMAs and commits
 // (multicast to both CTAs' barriers), warps 2-5 drain the CTA's own half of

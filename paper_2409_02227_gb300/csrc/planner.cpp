@@ -377,7 +377,8 @@ void finalize_schedule(goldy_schedule* s) {
     }
   }
   // fused schedules of several GEMMs keep 8 bytes per GEMM at the end of the
-  // workspace, reserved (part of the size goldy_schedule_query documents)
+  // workspace that nothing reads: the sizes that goldy_schedule_query documents
+  // stay as callers know them
   if ((s->flags & GOLDY_PLAN_FUSED) && s->gemms.size() > 1) off = align(off + 8 * s->gemms.size());
   s->workspace_bytes = off;
 }

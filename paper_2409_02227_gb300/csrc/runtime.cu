@@ -9,8 +9,8 @@
 // launch mode the GEMMs of a wave that share a kernel kind go out as one
 // persistent launch over all their tiles instead, and most plans of the dynamic
 // logic as one launch per kernel family (CTA pair, single CTA), output dtype and
-// 16 GEMMs, over the tiles of all its GEMMs.  The whole run can be captured once into a CUDA graph and replayed
-// with one launch.
+// 16 GEMMs, over the tiles of all its GEMMs.  The whole run can be captured once
+// into a CUDA graph and replayed with one launch.
 //
 // Per GEMM the host encodes two TMA tensor maps (A and B), sizes the
 // persistent grid as min(units, resident CTAs per SM * SMs / rc_div) — the
@@ -641,15 +641,15 @@ unsigned long long* trace_for(unsigned grid) {
 }
 
 // The kind that runs a launch planned for `kind` (an explicit schedule runs
-// the kinds it names).  With inputs_ready the next
-// run's CTAs may load and multiply while this run's wait for their stores, if
-// an SM has room for them: a launch of at most two CTAs' worth of units per SM
-// therefore takes the two-per-SM kind of the same tile shape (same K split,
-// same order of sums: the same bytes), so that a run no longer starts when the
-// one before leaves its SMs.  Measured back to back: four layers of eight 32 x
-// 4096 x 1024 59.6 -> 47.7 us, of four 128 x 1024 x 4096 split 4 41.8 -> 36.3
-// us, 753 x 1152 x 704 and a smaller one 6.7 -> 4.5 us, two 18 x 3904 x 896 3.5
-// -> 2.6 us.  K splits only when two runs do not fit side by side anyway: the
+// the kinds it names).  With inputs_ready the next run's CTAs may load and
+// multiply while this run's wait for their stores, if an SM has room for them: a
+// launch of at most two CTAs' worth of units per SM therefore takes the
+// two-per-SM kind of the same tile shape (same K split, same order of sums: the
+// same bytes), so that a run no longer starts when the one before leaves its
+// SMs.  Measured back to back: four layers of eight 32 x 4096 x 1024 54.3 ->
+// 42.2 us, of four 128 x 1024 x 4096 split 4 41.9 -> 36.4, two 18 x 3904 x 896
+// 3.3 -> 2.6 (a step alone pays for the shallower ring: 128 x 1024 x 4096 x 4
+// 17.2 -> 19.7 us).  K splits only when two runs do not fit side by side anyway: the
 // two-per-SM kinds have no room for pushed partials (two 256 x 256 x 512 split
 // 4, 64 CTAs: 3.06 -> 3.90 us), and 39 units of 31 K blocks lost 10%.  GEMMs of
 // different splits (split = 0) only with more units than SMs: 86 units of four
@@ -658,9 +658,9 @@ unsigned long long* trace_for(unsigned grid) {
 //
 // Without inputs_ready the same kind pays where one CTA per SM would leave a
 // second round for a few units: between one and two units per SM all of them
-// run at once (four layers of eight 32 x 4096 x 1024, 256 units: 64.5 -> 59.5
+// run at once (four layers of eight 32 x 4096 x 1024, 256 units: 64.3 -> 59.8
 // us; 777 x 1501 x 1003, 168 units: 12.6 -> 10.7; two 89 x 960 x 1984 split:
-// 14.5 -> 8.6).
+// 14.6 -> 8.5).
 //
 // `cap` is the planned kind's grid cap.  A launch that may not use the whole GPU
 // keeps its share: it takes the two-per-SM kind only where the cap does not bind
