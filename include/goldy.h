@@ -118,8 +118,8 @@ typedef struct goldy_graph goldy_graph;
  * alone, the largest first, each overlapping the previous one's tail.  Without
  * inputs_ready such a run starts after what was enqueued before it on the
  * streams that the separate launches would have used, and what is enqueued
- * there later starts after the run.  Two launches that run side by side or
- * whose K splits are reduced on chip may stay apart.  Without FUSED every GEMM
+ * there later starts after the run.  Launches that run side by side, and two
+ * whose K splits are reduced on chip, may stay apart.  Without FUSED every GEMM
  * is its own launch on its slot's stream and the groups run one after another.
  * The plan (groups, CDs, variants, slots) is the same, and so are the results,
  * byte for byte. */

@@ -1224,27 +1224,37 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
       apart = by_split.size() == 2;
       if (apart) sets.swap(by_split);
     }
-    // In a prepared run without inputs_ready, two launches on two streams also
-    // stay apart where they run side by side: all units fit on the GPU at once,
-    // or the pair launch needs no more rounds on the SMs that the other leaves.
-    // Joined, each replay waits for the second stream before it starts (see
-    // `ordered` below), which costs more than the second launch: 47 units in two
-    // launches 12.7 -> 10.3 us, 118 12.2 -> 10.3, 77 pair tiles and 36 units 22.5
-    // -> 20.5.  (A goldy_run is enqueued no faster than it runs, so that wait is
-    // over by then: 79 units joined 8.7 us, apart 11.4.)
-    if (!apart && t_rec && !t_early && sets.size() == 2 && (sets[0].slot | sets[1].slot) != 0 && !sets[0].degenerate &&
-        !sets[1].degenerate) {
-      int64_t units_of[2] = {0, 0}, sms_of[2];
-      bool pair[2];
-      for (int t = 0; t < 2; ++t) {
-        pair[t] = kKinds[s->gemms[sets[t].members[0]].kind].pair != 0;
-        for (int j = 0; j < sets[t].n; ++j) units_of[t] += s->gemms[sets[t].members[j]].units;
-        sms_of[t] = units_of[t] * (pair[t] ? 2 : 1);
+    // Without inputs_ready, launches on several streams also stay apart where
+    // they run side by side, all units on the GPU at once.  A joined pair launch
+    // and the other one follow each other (three launches, 96 SMs' worth of
+    // units: 21.6 -> 16.4 us; 144: 29.7 -> 24.6; 84: 21.1 -> 18.4), and each
+    // joined run waits for the other streams before it starts (see `ordered`
+    // below).  Two launches of single-CTA kinds: in a prepared run (47 units 12.7
+    // -> 10.3 us, 118 12.2 -> 10.3), and where K splits would reduce through the
+    // workspace (goldy_run, 47 units 12.2 -> 10.3, 115 15.5 -> 12.4; without
+    // splits one launch is enqueued sooner than two, 79 units 8.7 us against
+    // 11.4).  And in a prepared run a pair launch that needs no more rounds on the
+    // SMs that the other launch leaves (77 tiles and 36 units 22.5 -> 20.5).
+    if (!apart && !t_early && sets.size() > 1 && (slots & ~1u) != 0) {
+      int64_t sm_need = 0, others = 0;
+      const LaunchSet* pair = nullptr;
+      bool singles = false, split = false, empty = false;
+      for (const LaunchSet& ls : sets) {
+        const bool is_pair = !ls.degenerate && kKinds[s->gemms[ls.members[0]].kind].pair != 0;
+        empty = empty || ls.degenerate;
+        singles = singles || !is_pair;
+        if (is_pair) pair = &ls;
+        for (int j = 0; j < ls.n; ++j) {
+          const GemmPlan& gp = s->gemms[ls.members[j]];
+          sm_need += is_pair ? 2 * gp.units : gp.units;
+          if (!is_pair) others += gp.units;
+          split = split || gp.split > 1;
+        }
       }
-      apart = sms_of[0] + sms_of[1] <= sms(*d);
-      for (int t = 0; t < 2 && !apart; ++t)
-        apart = pair[t] && !pair[1 - t] && units_of[1 - t] < sms(*d) &&
-                pair_limit(s, sets[t].members, sets[t].n, units_of[1 - t], sms(*d)) > 0;
+      const bool two = sets.size() == 2;
+      apart = !empty && sm_need <= sms(*d) && ((pair && singles) || (two && (t_rec || split)));
+      if (!apart && !empty && two && t_rec && pair && singles && others < sms(*d))
+        apart = pair_limit(s, pair->members, pair->n, others, sms(*d)) > 0;
     }
   }
   const bool join_launches = fused && s->auto_plan && !apart && sets.size() > 1;

@@ -114,13 +114,14 @@ def test_mixed_launch_has_two_ctas_per_sm(cuda_ok, wide, out):
 @pytest.mark.parametrize("out", [F32, BF16])
 @pytest.mark.parametrize("ready", [False, True])
 def test_cluster_reduced_launches_stay_apart(cuda_ok, ready, out):
-    """Two launches of which K splits that clusters reduce are two thirds stay two; with less they join."""
+    """Two launches of which K splits that clusters reduce are two thirds stay two; with less they join, if with
+    inputs_ready."""
     # (M, N, K, kind, split): 48 of 59 units split 4; 32 of 43; two splits of one kind; 16 of 43; split 2
     for specs, want in (([(122, 1536, 2624, 2, 4), (38, 704, 256, 0, 1)], [48, 11]),
                         ([(122, 1024, 2624, 2, 4), (38, 704, 256, 0, 1)], [32, 11]),
                         ([(60, 1024, 1472, 8, 8), (41, 512, 1600, 8, 4)], [64, 16] if ready else [80]),
-                        ([(122, 512, 2624, 2, 4), (38, 1728, 256, 0, 1)], [43]),
-                        ([(122, 1536, 2624, 2, 2), (38, 704, 256, 0, 1)], [35])):
+                        ([(122, 512, 2624, 2, 4), (38, 1728, 256, 0, 1)], [43] if ready else [16, 27]),
+                        ([(122, 1536, 2624, 2, 2), (38, 704, 256, 0, 1)], [35] if ready else [24, 11])):
         shapes = [s[:3] for s in specs]
         entries, descs = [], []
         for M, N, K, kind, split in specs:
@@ -230,6 +231,22 @@ def test_mixed_launch_with_unaligned_batch_entries(cuda_ok, stride, per_sm):
     for e in range(batch - 1):                # nothing written between the entries
         assert bool((C0[e * stride + M * N:(e + 1) * stride] == -7.0).all())
     assert int(trace[12]) == min(192 + 16, per_sm * sms)
+
+
+@pytest.mark.parametrize("ready", [False, True])
+def test_launches_that_run_side_by_side_stay_apart(cuda_ok, ready):
+    """Pair tiles next to single-CTA kinds that all fit on the GPU at once: a launch each without inputs_ready,
+    one of the pair kernel and one of the others with it; with more tiles than fit, joined either way."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    small = [(100, 640, 1400, 2, 1), (40, 1280, 1200, 8, 1)]              # 5 and 10 units
+    for tiles_n, fits in (((sms - 15) // 4, True), ((sms - 15) // 4 + 2, False)):
+        specs = [(500, 256 * tiles_n - 64, 1096, 10, 1)] + small          # two rows of tiles
+        grids = sorted(len(u) for u in _units(specs, F32, inputs_ready=ready))
+        pair = min(4 * tiles_n, sms // 2 * 2)
+        if fits and not ready:
+            assert grids == sorted([pair, 5, 10])
+        else:
+            assert len(grids) == 2 and grids[0] == 15
 
 
 def test_long_pair_launch_takes_the_whole_gpu(cuda_ok):

@@ -54,13 +54,15 @@ def test_coruns_add_keeps_the_order_of_its_stream(cuda_ok, policy, prepared):
 
 
 # (M, N, K, kind): one launch each of a fused wave, so one stream each; the
-# first set's three kinds join into two launches, the second's into one
-WAVES = [[(100, 320, 1496, 2), (40, 1500, 1200, 8), (700, 600, 1096, 10)],
-         [(200, 320, 456, 2), (40, 300, 520, 8), (20, 600, 1000, 6)]]
+# first set's three kinds join into two launches, the second's into one, the
+# third's run side by side
+WAVES = [[(100, 320, 1496, 2), (40, 1500, 1200, 8), (2500, 2600, 1096, 10)],
+         [(200, 320, 456, 2), (40, 300, 520, 8), (20, 600, 1000, 6)],
+         [(100, 320, 1496, 2), (40, 1500, 1200, 8), (700, 600, 1096, 10)]]
 
 
 @pytest.mark.parametrize("how", ["run", "exec", "captured run", "captured exec"])
-@pytest.mark.parametrize("wave", [0, 1])
+@pytest.mark.parametrize("wave", [0, 1, 2])
 def test_joined_run_keeps_the_order_of_its_streams(cuda_ok, wave, how):
     specs = WAVES[wave]
     entries, descs = [], []
@@ -133,7 +135,7 @@ def test_joined_run_keeps_the_order_of_its_streams(cuda_ok, wave, how):
 def test_joined_run_reads_what_the_kernel_before_it_wrote(cuda_ok, how):
     """The later launches of a joined run start while its first is still going on; their operands, written by
     the kernel right before the run, have to be there all the same."""
-    specs = [(700, 2600, 1096, 10), (100, 1320, 4096, 2), (40, 1500, 2200, 8), (20, 600, 4000, 6)]
+    specs = [(2500, 2600, 1096, 10), (100, 1320, 4096, 2), (40, 1500, 2200, 8), (20, 600, 4000, 6)]
     entries, descs = [], []
     for M, N, K, kind in specs:
         d = G.desc(M, N, K, F32, lda=K, ldb=(N + 7) // 8 * 8, ldc=N)
