@@ -1210,6 +1210,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   uint32_t slots = 0;                        // the slots on whose streams these launches would go out
   for (const LaunchSet& ls : sets) slots |= 1u << ls.slot;
   bool apart = false;
+  int limit = 0;                             // CTAs of the run's one pair launch (see pair_limit); 0: no limit
   if (fused && s->auto_plan) {
     int64_t units = 0, reducible = 0;
     bool single = true;                      // single-CTA kinds only, nothing degenerate
@@ -1233,17 +1234,21 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
     // -> 10.3 us, 118 12.2 -> 10.3), and where K splits would reduce through the
     // workspace (goldy_run, 47 units 12.2 -> 10.3, 115 15.5 -> 12.4; without
     // splits one launch is enqueued sooner than two, 79 units 8.7 us against
-    // 11.4).  And in a prepared run a pair launch that needs no more rounds on the
-    // SMs that the other launch leaves (77 tiles and 36 units 22.5 -> 20.5).
+    // 11.4).  And a pair launch that needs no more rounds on the SMs that the
+    // others leave (77 tiles and 36 units 22.5 -> 20.5; 85 and 43 units in three
+    // launches 25.8 -> 20.6; goldy_run, 100 and 27 19.2 -> 16.6).
     if (!apart && !t_early && sets.size() > 1 && (slots & ~1u) != 0) {
       int64_t sm_need = 0, others = 0;
       const LaunchSet* pair = nullptr;
-      bool singles = false, split = false, empty = false;
+      bool singles = false, split = false, empty = false, one_pair = true;
       for (const LaunchSet& ls : sets) {
         const bool is_pair = !ls.degenerate && kKinds[s->gemms[ls.members[0]].kind].pair != 0;
         empty = empty || ls.degenerate;
         singles = singles || !is_pair;
-        if (is_pair) pair = &ls;
+        if (is_pair) {
+          one_pair = !pair;
+          pair = &ls;
+        }
         for (int j = 0; j < ls.n; ++j) {
           const GemmPlan& gp = s->gemms[ls.members[j]];
           sm_need += is_pair ? 2 * gp.units : gp.units;
@@ -1251,10 +1256,11 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
           split = split || gp.split > 1;
         }
       }
-      const bool two = sets.size() == 2;
-      apart = !empty && sm_need <= sms(*d) && ((pair && singles) || (two && (t_rec || split)));
-      if (!apart && !empty && two && t_rec && pair && singles && others < sms(*d))
-        apart = pair_limit(s, pair->members, pair->n, others, sms(*d)) > 0;
+      apart = !empty && sm_need <= sms(*d) && ((pair && singles) || (sets.size() == 2 && (t_rec || split)));
+      if (!apart && !empty && pair && one_pair && singles && others < sms(*d)) {
+        limit = 2 * pair_limit(s, pair->members, pair->n, others, sms(*d));
+        apart = limit > 0;
+      }
     }
   }
   const bool join_launches = fused && s->auto_plan && !apart && sets.size() > 1;
@@ -1367,6 +1373,7 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
             (sm_use(mid) <= double(sms(*d)) ? lo : hi) = mid;
           }
           fit = lo;
+          if (!join_launches) limit = 0;   // resident together without the limit
         }
       }
       for (size_t t = t0; t < t1; ++t) {
@@ -1465,7 +1472,6 @@ static goldy_status run_impl(const goldy_schedule* s, const void* const* A, cons
   // caller's own wait limit, which would come to cover the launch before.)
   const bool chain = one_stream && !t_early && join_launches && t_pdl && !t_trace && t_wait_ns == 0;
   bool chained = false;
-  int limit = 0;                             // CTAs of the pair launch (see pair_limit)
   if (join_launches && one_stream) {
     int64_t others = 0;
     const LaunchSet* pair = nullptr;
